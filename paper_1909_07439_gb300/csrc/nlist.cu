@@ -35,6 +35,7 @@ namespace sph {
 constexpr int kNlTB = 8;        // targets per candidate test batch
 constexpr int kNlWarps = 4;     // warps per block
 constexpr int kSG = 8;          // consecutive groups that may share one tree walk
+constexpr int kGrabs = 4;       // grabs per warp of the launch at least (fewer groups each in a small tree)
 constexpr int kSGLeaves = 320;  // leaves one walk may find
 constexpr int kMaxRuns = 128;   // candidate runs of one group (plus a sentinel)
 constexpr int kLWWide = 2;      // nodes per lane and walk step
@@ -295,13 +296,21 @@ __global__ void __launch_bounds__(kNlWarps * 32, 7) nlist_kernel(NlistArgs a)
     // per-warp tallies (32 bits: a warp's share of a launch stays far below 2^32)
     unsigned n_cand = 0, n_entries = 0, n_over = 0;
 
+    // A grab is one serial chain of walks, selections and tests of a warp, so a
+    // small tree is cut into grabs of fewer groups: kGrabs of them per warp of
+    // the launch, down to one group.  (With 8 groups whatever the tree's size, 2003
+    // particles kept 80 of 4256 warps busy: list build 101 -> 33 us; 8192 particles
+    // 147 -> 35 us, the M6 tube of 166 k 349 -> 241 us, 64^3 226 -> 210 us; from
+    // about 140 k groups on nothing changes.  1 to 8 grabs per warp measured alike,
+    // but for 1 at the tube: 283 us.)
+    const int most = min(kSG, max(1, ng / (kGrabs * (int)gridDim.x * kNlWarps)));
     while (true) {
         // kSG groups at a time, kSG / 2 in the last quarter (shorter tail);
         // with a due mask (block steps) kSG / 2 throughout: the due groups are
         // few and clustered, and smaller grabs spread them over more warps
-        int gf = 0, grab = kSG;
+        int gf = 0, grab = most;
         if (lane == 0) {
-            grab = a.active || *(volatile int *)a.work >= ng - (ng >> 2) ? kSG / 2 : kSG;
+            grab = min(most, a.active || *(volatile int *)a.work >= ng - (ng >> 2) ? kSG / 2 : kSG);
             gf = atomicAdd(a.work, grab);
         }
         gf = __shfl_sync(0xffffffffu, gf, 0);
