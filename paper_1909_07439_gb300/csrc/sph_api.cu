@@ -152,7 +152,6 @@ sph_status check_params(Ctx &c, const sph_params *p)
         if (e_ != cudaSuccess) return cuda_fail(c, e_, what); \
     } while (0)
 
-constexpr int kTreeLaunches = 33;
 constexpr int kPrepLaunches = 1;
 
 // tree_fresh: the tree was just built from this state (node and group h_max
@@ -163,7 +162,7 @@ sph_status do_density(Ctx &c, const sph_state &s, const sph_params &p, cudaStrea
 {
     if (!tree_fresh) {
         // node and group h_max of the starting h, for the list walk
-        StageScope sc(c, ST_PREP, st, 3);
+        StageScope sc(c, ST_PREP, st, 2);
         CK(update_hmax(c, s, p, st), "update_hmax");
         CK(pack_records(c, s, st), "pack");
     }
@@ -187,8 +186,8 @@ sph_status do_force(Ctx &c, const sph_state &s, const sph_params &p, cudaStream_
         if (!records_fresh) CK(pack_records(c, s, st), "pack");
     }
     {
-        // relist (h_max refresh 2, list kernel 1), list kernel, h_max refresh 2, walking fallback
-        StageScope sc(c, ST_FORCE, st, 7);
+        // relist (h_max refresh, list kernel), list kernel, h_max refresh, walking fallback
+        StageScope sc(c, ST_FORCE, st, 5);
         CK(force_pass(c, s, p, st), "force");
     }
     if (p.grav_G > 0.f) {
@@ -200,7 +199,7 @@ sph_status do_force(Ctx &c, const sph_state &s, const sph_params &p, cudaStream_
 
 sph_status do_tree(Ctx &c, const sph_state &s, const sph_params &p, bool full, cudaStream_t st)
 {
-    StageScope sc(c, ST_TREE, st, kTreeLaunches);
+    StageScope sc(c, ST_TREE, st, tree_launches(s.n, full));
     CK(build_tree(c, s, p, full, st), "build_tree");
     return SPH_OK;
 }
@@ -417,7 +416,6 @@ sph_status sph_create(sph_ctx **out, int64_t max_n, int device)
     A(dalloc(t.node_lo, t.cap_nodes));
     A(dalloc(t.node_hi, t.cap_nodes));
     A(dalloc(t.node_ref, t.cap_nodes));
-    A(dalloc(t.level_start, kLevels + 1));
     A(dalloc(t.grp_ref, t.cap_groups));
     A(dalloc(t.grp_lo, t.cap_groups));
     A(dalloc(t.grp_hi, t.cap_groups));
@@ -473,7 +471,7 @@ void sph_destroy(sph_ctx *h)
                     c.tmp4[3], c.tmp1[0], c.tmp1[1], c.tmp1[2], c.tmp1[3], c.tmp1[4], c.tmp_perm,
                     c.tree.node_first, c.tree.node_count, c.tree.node_level, c.tree.node_child,
                     c.tree.node_nchild, c.tree.node_parent, c.tree.node_arrive, c.tree.node_lo,
-                    c.tree.node_hi, c.tree.node_ref, c.tree.level_start, c.tree.grp_ref,
+                    c.tree.node_hi, c.tree.node_ref, c.tree.grp_ref,
                     c.tree.grp_lo, c.tree.grp_hi, c.tree.lv_tree, c.tree.lv_grp, c.tree.blk_cnt,
                     c.nl_idx, c.nl_len, c.fallback,
                     c.tree.rec_ctl, c.tree.rec_bad,
@@ -588,7 +586,7 @@ sph_status sph_step_block(sph_ctx *h, sph_state *s, const sph_params *p, int max
             CK(block_substep(c, *s, *p, d_level, j, max_level, d_dt_min, st), "block substep");
         }
         {
-            StageScope sc(c, ST_TREE, st, 2);
+            StageScope sc(c, ST_TREE, st, 1);
             CK(refit_tree(c, *s, st), "refit");
         }
         c.mask = c.active;

@@ -73,7 +73,6 @@ struct Tree {
     float4 *node_lo = nullptr;   // x, y, z, h_max
     float4 *node_hi = nullptr;   // x, y, z, unused
     int2 *node_ref = nullptr;    // leaf: (first, count); internal: (child_first, -nchild)
-    int *level_start = nullptr;  // [kLevels + 1]
     // groups: terminal nodes of the n_group chop
     int2 *grp_ref = nullptr;     // (first, count)
     float4 *grp_lo = nullptr;    // x, y, z, h_max
@@ -225,6 +224,8 @@ inline float3 box_lo_of(const sph_params &p) { return make_float3(p.box_lo[0], p
 // tree.cu
 cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool full_permute,
                        cudaStream_t st, const Batch *batch = nullptr);
+// kernels that build_tree launches for n particles (without a batch)
+int tree_launches(int64_t n, bool full_permute);
 cudaError_t instance_map(Ctx &c, const int64_t *d_offsets, int n_inst, int n, cudaStream_t st);
 // node and group h_max of the current h; gate != nullptr: only if *gate != 0
 cudaError_t update_hmax(Ctx &c, const sph_state &s, const sph_params &p, cudaStream_t st,

@@ -439,6 +439,56 @@ __global__ void rs_fixup_kernel(uint64_t *keys, uint32_t *vals, int n, int *full
     }
 }
 
+// Few particles: the slot of each key is the number of keys before it, counted
+// by comparing it with all others.  One kernel of n^2 comparisons over all SMs
+// takes the place of the radix sort's 17 launches and their chain of single-block
+// passes; the order is that of the stable sort by (instance, key, input slot).
+// A block ranks kRankE keys, kRankP threads each, against tiles of all keys in
+// shared memory.  2003 keys 8 us, 8192 keys 25 us, against 66 us for the radix
+// sort of either; the comparisons grow with n^2.
+constexpr int kRankSort = 8192;  // particles at most
+constexpr int kRankE = 32, kRankP = 8, kRankTile = 1024;
+template <bool BATCH>
+__global__ void __launch_bounds__(kRankE * kRankP) rank_sort_kernel(const uint64_t *__restrict__ keys,
+                                                                    const int *__restrict__ inst, int n,
+                                                                    uint64_t *__restrict__ kout,
+                                                                    uint32_t *__restrict__ order)
+{
+    __shared__ uint64_t sk[kRankTile];
+    __shared__ int si[BATCH ? kRankTile : 1];
+    const int part = threadIdx.x & (kRankP - 1);
+    const int i0 = blockIdx.x * kRankE, i = i0 + threadIdx.x / kRankP;
+    const bool valid = i < n;
+    const uint64_t key = valid ? keys[i] : 0;
+    const int own = BATCH && valid ? inst[i] : 0;
+    int rank = 0;
+    for (int t0 = 0; t0 < n; t0 += kRankTile) {
+        const int cnt = min(kRankTile, n - t0);
+        __syncthreads();
+        for (int m = threadIdx.x; m < cnt; m += kRankE * kRankP) {
+            sk[m] = keys[t0 + m];
+            if (BATCH) si[m] = inst[t0 + m];
+        }
+        __syncthreads();
+        if (BATCH || (t0 < i0 + kRankE && i0 < t0 + kRankTile)) {
+            for (int m = part; m < cnt; m += kRankP) {
+                bool before = sk[m] < key || (sk[m] == key && t0 + m < i);
+                if (BATCH) before = si[m] < own || (si[m] == own && before);
+                rank += before ? 1 : 0;
+            }
+        } else {  // a tile of earlier slots only, or of later ones only
+            const uint64_t below = key + (t0 < i0 ? 1 : 0);  // keys have 63 bits
+#pragma unroll 4
+            for (int m = part; m < cnt; m += kRankP) rank += sk[m] < below ? 1 : 0;
+        }
+    }
+    for (int o = kRankP / 2; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (valid && part == 0) {
+        kout[rank] = key;
+        order[rank] = (uint32_t)i;
+    }
+}
+
 // ------------------------------------------------------------------ gather
 struct GatherArgs {
     const uint32_t *order;
@@ -470,6 +520,20 @@ __global__ void gather_kernel(GatherArgs g, int n)
             if (a < g.n1) g.t1[a][k] = g.a1[a][o];
         g.tperm[k] = g.perm[o];
         if (g.keys_sorted) g.keys_out[k] = g.keys_sorted[k];
+    }
+}
+
+// the gathered arrays back into the state (one launch for all of them)
+__global__ void copy_back_kernel(GatherArgs g, int n)
+{
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            if (a < g.n4) g.a4[a][k] = g.t4[a][k];
+#pragma unroll
+        for (int a = 0; a < 5; ++a)
+            if (a < g.n1) g.a1[a][k] = g.t1[a][k];
+        g.perm[k] = g.tperm[k];
     }
 }
 
@@ -509,8 +573,10 @@ __global__ void __launch_bounds__(SC_T) scan_part_kernel(int *part, int nb, int 
     if (threadIdx.x == 0 && total) *total = (int)carry;
 }
 
+// starts != nullptr: (i, 0) into starts[out value] for every counted i, in
+// place of the values
 __global__ void __launch_bounds__(SC_T) scan_down_kernel(const int *in, int *out, int n, int mode,
-                                                         const int *part)
+                                                         const int *part, int2 *starts)
 {
     __shared__ uint32_t ws[8];
     int base = blockIdx.x * SC_CHUNK + threadIdx.x * SC_I;
@@ -522,19 +588,68 @@ __global__ void __launch_bounds__(SC_T) scan_down_kernel(const int *in, int *out
     int run = part[blockIdx.x] + (int)ex;
 #pragma unroll
     for (int k = 0; k < SC_I; ++k)
-        if (base + k < n) { out[base + k] = run; run += v[k]; }
+        if (base + k < n) {
+            if (!starts) out[base + k] = run;
+            else if (v[k]) starts[run] = make_int2(base + k, 0);
+            run += v[k];
+        }
+}
+
+// The whole scan by one block, 8 entries per thread at a time: up to one round
+// it costs less than two more launches (3.8 us against 9.3 us in three kernels;
+// four rounds, at 30 k entries, take 15 us).
+constexpr int SC1_T = 1024, kScanOne = SC1_T * SC_I;
+__global__ void __launch_bounds__(SC1_T) scan_one_kernel(const int *in, int *out, int n, int mode,
+                                                         int *total, int2 *starts)
+{
+    __shared__ int ws[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int carry = 0;
+    for (int b = 0; b < n; b += SC1_T * SC_I) {
+        const int base = b + threadIdx.x * SC_I;
+        int v[SC_I], s = 0;
+#pragma unroll
+        for (int k = 0; k < SC_I; ++k) { v[k] = scan_in(in, base + k, n, mode); s += v[k]; }
+        int x = s;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) ws[w] = x;
+        __syncthreads();
+        int t = ws[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        const int before = __shfl_sync(0xffffffffu, t, w > 0 ? w - 1 : 0);
+        int run = carry + (w > 0 ? before : 0) + x - s;
+        carry += __shfl_sync(0xffffffffu, t, 31);
+#pragma unroll
+        for (int k = 0; k < SC_I; ++k)
+            if (base + k < n) {
+                if (!starts) out[base + k] = run;
+                else if (v[k]) starts[run] = make_int2(base + k, 0);
+                run += v[k];
+            }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0 && total) *total = carry;
 }
 
 // mode 0: out[i] = sum_{k<i} in[k]; mode 1: counts in[k] >= 0
 static cudaError_t scan_mode(Ctx &c, const int *in, int *out, int n, int mode, int *total_dev,
-                             cudaStream_t st)
+                             cudaStream_t st, int2 *starts = nullptr)
 {
+    if (n <= kScanOne) {
+        scan_one_kernel<<<1, SC1_T, 0, st>>>(in, out, n, mode, total_dev, starts);
+        return cudaGetLastError();
+    }
     int nb = div_up(n, SC_CHUNK);
-    if (nb < 1) nb = 1;
     if (nb > c.scan_part_cap) return cudaErrorInvalidValue;
     scan_reduce_kernel<<<nb, SC_T, 0, st>>>(in, n, mode, c.scan_part);
     scan_part_kernel<<<1, SC_T, 0, st>>>(c.scan_part, nb, total_dev);
-    scan_down_kernel<<<nb, SC_T, 0, st>>>(in, out, n, mode, c.scan_part);
+    scan_down_kernel<<<nb, SC_T, 0, st>>>(in, out, n, mode, c.scan_part, starts);
     return cudaGetLastError();
 }
 
@@ -570,13 +685,15 @@ __device__ __forceinline__ int cd_slots(const uint64_t *__restrict__ keys,
 // T slots: Lmax = max(d, min(q[s] + 1, kMaxLevel)).  b[s] = -1 is a root
 // (d = 0), b[s] = kMaxLevel a key equal to the previous one (no node).
 //
-// One block per tile of kCfTile slots, with halos of kCfHalo > T slots on
-// both sides in shared memory (one byte per slot); the window minima and
-// maxima by doubling.
-constexpr int kCfTile = 2048, kCfHalo = 65, kCfR = kCfTile + 2 * kCfHalo;
+// One block per tile of TILE slots, with halos of kCfHalo > T slots on both
+// sides in shared memory (one byte per slot); the window minima and maxima by
+// doubling.  Tiles of kCfTile slots; of kCfSmall where those would leave SMs
+// without a block (a block's passes are a chain of
+// barriers: 2003 slots 15.4 -> 5.5 us, 64^3 16 -> 9 us).
+constexpr int kCfTile = 2048, kCfSmall = 256, kCfHalo = 65;
 
 // dst[i] = min (or max) of src[i + off .. i + off + len - 1] for i in [lo, hi);
-// needs lo + off >= 0 and hi + off + len <= kCfR, and reads src only there.
+// needs lo + off >= 0 and hi + off + len <= TILE + 2 kCfHalo, and reads src only there.
 // t0, t1: scratch.
 template <bool MAX>
 __device__ __forceinline__ void cf_window(const signed char *src, signed char *dst, signed char *t0,
@@ -603,17 +720,19 @@ __device__ __forceinline__ void cf_window(const signed char *src, signed char *d
     __syncthreads();
 }
 
+template <int TILE>
 __global__ void __launch_bounds__(256) chop_flags_kernel(const uint64_t *__restrict__ keys,
                                                          const int *__restrict__ inst, int n,
                                                          int t_leaf, int t_group, int *lv_tree,
                                                          int *lv_grp)
 {
     // local index i <-> slot t0 - kCfHalo + i
-    __shared__ signed char sb[kCfR], sq[kCfR], sm[kCfR], s0[kCfR], s1[kCfR];
-    const int ntile = (n + kCfTile - 1) / kCfTile;
+    constexpr int R = TILE + 2 * kCfHalo;
+    __shared__ signed char sb[R], sq[R], sm[R], s0[R], s1[R];
+    const int ntile = (n + TILE - 1) / TILE;
     for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
-        const int t0 = tile * kCfTile;
-        for (int i = threadIdx.x; i < kCfR; i += blockDim.x) {
+        const int t0 = tile * TILE;
+        for (int i = threadIdx.x; i < R; i += blockDim.x) {
             const int x = t0 - kCfHalo + i;
             sb[i] = (signed char)(x <= 0 || x >= n ? -1 : cd_slots(keys, inst, x - 1, x));
         }
@@ -622,11 +741,11 @@ __global__ void __launch_bounds__(256) chop_flags_kernel(const uint64_t *__restr
             const int T = pass == 0 ? t_leaf : t_group;
             int *lv = pass == 0 ? lv_tree : lv_grp;
             if (pass == 0 || t_group != t_leaf) {
-                // q over [-T, kCfTile) relative to t0, then the maxima over [s - T, s]
-                cf_window<false>(sb, sq, s0, s1, kCfHalo - T, kCfHalo + kCfTile, 1, T);
-                cf_window<true>(sq, sm, s0, s1, kCfHalo, kCfHalo + kCfTile, -T, T + 1);
+                // q over [-T, TILE) relative to t0, then the maxima over [s - T, s]
+                cf_window<false>(sb, sq, s0, s1, kCfHalo - T, kCfHalo + TILE, 1, T);
+                cf_window<true>(sq, sm, s0, s1, kCfHalo, kCfHalo + TILE, -T, T + 1);
             }
-            for (int k = threadIdx.x; k < kCfTile && t0 + k < n; k += blockDim.x) {
+            for (int k = threadIdx.x; k < TILE && t0 + k < n; k += blockDim.x) {
                 const int i = kCfHalo + k;
                 const int bs = sb[i], qs = sq[i];
                 int v;
@@ -688,9 +807,10 @@ __global__ void __launch_bounds__(256) chop_count_kernel(const int *__restrict__
 // warps, then per warp and level the ballots again for the ranks.
 __global__ void __launch_bounds__(256) chop_write_kernel(const int *__restrict__ lv, int n,
                                                          const int *__restrict__ blk_off, int nb,
-                                                         Tree t, int *err)
+                                                         const int *total, Tree t, int *sizes, int *err)
 {
     __shared__ int wcnt[kLevels][8];
+    if (blockIdx.x == 0 && threadIdx.x == 0) sizes[SZ_NODES] = min(*total, t.cap_nodes);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int base = blockIdx.x * kChopBlock + w * 32 * kCwR;
@@ -735,17 +855,6 @@ __global__ void __launch_bounds__(256) chop_write_kernel(const int *__restrict__
     }
 }
 
-__global__ void level_start_kernel(const int *blk_off, int nb, const int *total, Tree t,
-                                   int *sizes)
-{
-    int L = threadIdx.x;
-    if (L < kLevels) t.level_start[L] = blk_off[L * nb];
-    if (L == kLevels) {
-        t.level_start[kLevels] = *total;
-        sizes[SZ_NODES] = min(*total, t.cap_nodes);
-    }
-}
-
 // end of the run at level L that starts at s (galloping search).  The
 // root run of a batch instance is its slots (the sort keeps each instance's
 // slots together), found from the instance ids, so the tree stays inside
@@ -768,9 +877,12 @@ __device__ int run_end(const uint64_t *__restrict__ keys, const int *__restrict_
 }
 
 __global__ void node_finish_kernel(const uint64_t *__restrict__ keys, const int *__restrict__ inst,
-                                   int n, int T, Tree t, const int *sizes)
+                                   int n, int T, const int *__restrict__ blk_off, int nb, Tree t,
+                                   const int *sizes)
 {
-    int nn = sizes[SZ_NODES];
+    const int nn = sizes[SZ_NODES];
+    // first node of level L (blk_off: the nodes per level and block, scanned)
+    auto level_start = [&](int L) { return L < kLevels ? min(blk_off[L * nb], nn) : nn; };
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nn; k += gridDim.x * blockDim.x) {
         int L = t.node_level[k], s = t.node_first[k];
         int cnt = run_end(keys, inst, n, s, L) - s;
@@ -778,13 +890,13 @@ __global__ void node_finish_kernel(const uint64_t *__restrict__ keys, const int 
         if (L == 0) t.node_parent[k] = -1;
         int cf = -1, nc = 0;
         if (cnt > T && L < kMaxLevel) {
-            int lo = t.level_start[L + 1], hi = min(t.level_start[L + 2], nn);
+            const int e = level_start(L + 2);
+            int lo = level_start(L + 1), hi = e;
             while (lo < hi) {
                 int mid = (lo + hi) >> 1;
                 if (t.node_first[mid] < s) lo = mid + 1; else hi = mid;
             }
             cf = lo;
-            int e = min(t.level_start[L + 2], nn);
             while (cf + nc < e && t.node_first[cf + nc] < s + cnt) {
                 t.node_parent[cf + nc] = k;
                 ++nc;
@@ -798,14 +910,11 @@ __global__ void node_finish_kernel(const uint64_t *__restrict__ keys, const int 
 
 // Bottom-up bounds: leaves from particles, parents from children; the last
 // child to finish (arrival counter, reset by that child) computes its parent.
-// gate != nullptr: do nothing unless *gate != 0.  what = 0: AABB of
-// positions and h_max; what = 1: h_max only.
-__global__ void node_bounds_kernel(const float4 *__restrict__ pos, const float *__restrict__ h,
-                                   Tree t, const int *sizes, int what, const int *gate)
+// what = 0: AABB of positions and h_max; what = 1: h_max only.
+__device__ __forceinline__ void node_bounds(const float4 *__restrict__ pos, const float *__restrict__ h,
+                                            const Tree &t, int nn, int what, int block, int blocks)
 {
-    if (gate && *gate == 0) return;
-    int nn = sizes[SZ_NODES];
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nn; k += gridDim.x * blockDim.x) {
+    for (int k = block * blockDim.x + threadIdx.x; k < nn; k += blocks * blockDim.x) {
         if (t.node_nchild[k] != 0) continue;
         int s = t.node_first[k], e = s + t.node_count[k];
         if (what == 0) {
@@ -857,21 +966,11 @@ __global__ void node_bounds_kernel(const float4 *__restrict__ pos, const float *
     }
 }
 
-// groups: first particle of each terminal node of the group chop
-__global__ void group_write_kernel(const int *__restrict__ lv_grp, const int *__restrict__ gidx,
-                                   int n, Tree t)
-{
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x)
-        if (lv_grp[s] >= 0) t.grp_ref[gidx[s]] = make_int2(s, 0);
-}
-
 // what = 0: count + AABB (h_max too); what = 1: h_max only
-__global__ void group_bounds_kernel(const float4 *__restrict__ pos, const float *__restrict__ h,
-                                    int n, Tree t, const int *sizes, int what, const int *gate)
+__device__ __forceinline__ void group_bounds(const float4 *__restrict__ pos, const float *__restrict__ h,
+                                             int n, const Tree &t, int ng, int what, int block, int blocks)
 {
-    if (gate && *gate == 0) return;
-    int ng = sizes[SZ_GROUPS];
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) {
+    for (int g = block * blockDim.x + threadIdx.x; g < ng; g += blocks * blockDim.x) {
         int s = t.grp_ref[g].x;
         int e = g + 1 < ng ? t.grp_ref[g + 1].x : n;
         float hm = 0.f;
@@ -892,6 +991,18 @@ __global__ void group_bounds_kernel(const float4 *__restrict__ pos, const float 
             t.grp_lo[g].w = hm;
         }
     }
+}
+
+// Bounds of the nodes (the first nb_nodes blocks) and of the groups (the
+// rest): independent of each other, one launch for both.  gate != nullptr: do
+// nothing unless *gate != 0.
+__global__ void __launch_bounds__(128) bounds_kernel(const float4 *__restrict__ pos, const float *__restrict__ h,
+                                                     int n, Tree t, const int *sizes, int what, const int *gate,
+                                                     int nb_nodes)
+{
+    if (gate && *gate == 0) return;
+    if ((int)blockIdx.x < nb_nodes) node_bounds(pos, h, t, sizes[SZ_NODES], what, blockIdx.x, nb_nodes);
+    else group_bounds(pos, h, n, t, sizes[SZ_GROUPS], what, blockIdx.x - nb_nodes, gridDim.x - nb_nodes);
 }
 
 // inst[k] = instance owning slot k (offsets ascending, every instance non-empty)
@@ -957,14 +1068,27 @@ cudaError_t instance_map(Ctx &c, const int64_t *d_offsets, int n_inst, int n, cu
     return cudaGetLastError();
 }
 
+// nodes that n particles can have (the context's capacity is for max_n)
+static int64_t node_cap_for(const Tree &t, int64_t n) { return std::min<int64_t>(t.cap_nodes, 2 * n + 1024); }
+
+static cudaError_t launch_bounds(Ctx &c, const sph_state &s, int what, const int *gate, cudaStream_t st)
+{
+    const int nb = grid_for(c, node_cap_for(c.tree, s.n), 128), gb = grid_for(c, s.n, 128);
+    bounds_kernel<<<nb + gb, 128, 0, st>>>((const float4 *)s.pos, s.h, (int)s.n, c.tree, c.d_sizes, what, gate, nb);
+    return cudaGetLastError();
+}
+
 cudaError_t refit_tree(Ctx &c, const sph_state &s, cudaStream_t st)
 {
-    const int n = (int)s.n;
-    Tree &t = c.tree;
-    const float4 *pos = (const float4 *)s.pos;
-    group_bounds_kernel<<<grid_for(c, n, 128), 128, 0, st>>>(pos, s.h, n, t, c.d_sizes, 0, nullptr);
-    node_bounds_kernel<<<grid_for(c, t.cap_nodes, 128), 128, 0, st>>>(pos, s.h, t, c.d_sizes, 0, nullptr);
-    return cudaGetLastError();
+    return launch_bounds(c, s, 0, nullptr, st);
+}
+
+int tree_launches(int64_t n, bool full)
+{
+    // box (2), keys, sort, gather (and copy back), chop flags, scans, counts, nodes (2), bounds
+    const int sort = n <= kRankSort ? 1 : 2 + 4 + 1 + 8;
+    const int scans = (n <= kScanOne ? 1 : 3) + (kLevels * (int64_t)div_up(n, kChopBlock) <= kScanOne ? 1 : 3);
+    return 3 + sort + 2 + (full ? 1 : 0) + scans + 4;
 }
 
 cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool full_permute,
@@ -992,39 +1116,48 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
     // 2. keys
     morton_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(pos_in, inst, n, bb, s.keys, c.idx_a,
                                                       period_of(p), box_lo_of(p), c.d_err);
-    // 3. radix sort (key, slot); a batch adds stable passes on the instance id,
-    //    which puts every instance back on its own slots
-    const int ntiles = div_up(n, RS_TILE);
+    // 3. sort (key, slot): few particles by counting ranks, else the radix sort,
+    //    where a batch adds stable passes on the instance id, which put every
+    //    instance back on its own slots
     uint64_t *kin = s.keys, *kout = c.keys_alt;
     uint32_t *vin = c.idx_a, *vout = c.idx_b;
-    const int ndigit = batch ? 10 : 8;  // digits 0..7 of the key, 8..9 of the instance id
-    const int nslot = 4 + 8 + (batch ? 2 : 0);
-    int *full = c.rs_tiles + kRsSlots;  // the fix-up found a long run: sort all 64 bits
-    // digit counts of all passes, their scans, fresh look-back words, tile counters, flag
-    SPH_TRY(cudaMemsetAsync(c.rs_ghist, 0, sizeof(uint32_t) * 10 * 256, st));
-    SPH_TRY(cudaMemsetAsync(c.rs_tiles, 0, sizeof(int) * (kRsSlots + 1), st));
-    SPH_TRY(cudaMemsetAsync(c.rs_status, 0, sizeof(uint32_t) * 256 * (size_t)ntiles * nslot, st));
-    const int gh_grid = (int)std::max<int64_t>(1, std::min<int64_t>(div_up(n, 256 * RS_GE), 4 * (int64_t)c.num_sms));
-    rs_ghist_kernel<<<gh_grid, 256, 0, st>>>(kin, inst, n, c.rs_ghist);
-    rs_gscan_kernel<<<ndigit, 256, 0, st>>>(c.rs_ghist, c.rs_gstart);
-    int slot = 0;
-    auto pass = [&](int digit, const int *gate) {
-        const int *dinst = digit >= 8 ? inst : nullptr;
-        const int shift = digit >= 8 ? 8 * (digit - 8) : 8 * digit;
-        rs_onesweep_kernel<<<ntiles, RS_T, 0, st>>>(kin, vin, kout, vout, dinst, n, shift,
-                                                    c.rs_gstart + 256 * digit,
-                                                    c.rs_status + (size_t)256 * ntiles * slot,
-                                                    c.rs_tiles + slot, c.d_err, gate, RS_SPIN);
-        ++slot;
-        std::swap(kin, kout);  // a gated pass that returns moves nothing, but
-        std::swap(vin, vout);  // the gated passes come in an even number
-    };
-    for (int digit = 4; digit < 8; ++digit) pass(digit, nullptr);
-    rs_fixup_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(kin, vin, n, full);
-    for (int digit = 0; digit < 8; ++digit) pass(digit, full);
-    if (batch) {
-        pass(8, nullptr);
-        pass(9, nullptr);
+    if (n <= kRankSort) {
+        const int grid = div_up(n, kRankE);
+        if (batch) rank_sort_kernel<true><<<grid, kRankE * kRankP, 0, st>>>(kin, inst, n, kout, vout);
+        else rank_sort_kernel<false><<<grid, kRankE * kRankP, 0, st>>>(kin, nullptr, n, kout, vout);
+        std::swap(kin, kout);
+        std::swap(vin, vout);
+    } else {
+        const int ntiles = div_up(n, RS_TILE);
+        const int ndigit = batch ? 10 : 8;  // digits 0..7 of the key, 8..9 of the instance id
+        const int nslot = 4 + 8 + (batch ? 2 : 0);
+        int *full = c.rs_tiles + kRsSlots;  // the fix-up found a long run: sort all 64 bits
+        // digit counts of all passes, their scans, fresh look-back words, tile counters, flag
+        SPH_TRY(cudaMemsetAsync(c.rs_ghist, 0, sizeof(uint32_t) * 10 * 256, st));
+        SPH_TRY(cudaMemsetAsync(c.rs_tiles, 0, sizeof(int) * (kRsSlots + 1), st));
+        SPH_TRY(cudaMemsetAsync(c.rs_status, 0, sizeof(uint32_t) * 256 * (size_t)ntiles * nslot, st));
+        const int gh_grid = (int)std::max<int64_t>(1, std::min<int64_t>(div_up(n, 256 * RS_GE), 4 * (int64_t)c.num_sms));
+        rs_ghist_kernel<<<gh_grid, 256, 0, st>>>(kin, inst, n, c.rs_ghist);
+        rs_gscan_kernel<<<ndigit, 256, 0, st>>>(c.rs_ghist, c.rs_gstart);
+        int slot = 0;
+        auto pass = [&](int digit, const int *gate) {
+            const int *dinst = digit >= 8 ? inst : nullptr;
+            const int shift = digit >= 8 ? 8 * (digit - 8) : 8 * digit;
+            rs_onesweep_kernel<<<ntiles, RS_T, 0, st>>>(kin, vin, kout, vout, dinst, n, shift,
+                                                        c.rs_gstart + 256 * digit,
+                                                        c.rs_status + (size_t)256 * ntiles * slot,
+                                                        c.rs_tiles + slot, c.d_err, gate, RS_SPIN);
+            ++slot;
+            std::swap(kin, kout);  // a gated pass that returns moves nothing, but
+            std::swap(vin, vout);  // the gated passes come in an even number
+        };
+        for (int digit = 4; digit < 8; ++digit) pass(digit, nullptr);
+        rs_fixup_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(kin, vin, n, full);
+        for (int digit = 0; digit < 8; ++digit) pass(digit, full);
+        if (batch) {
+            pass(8, nullptr);
+            pass(9, nullptr);
+        }
     }
     // the sorted (key, slot) pairs are in (kin, vin)
     // 4. permute the state into curve order
@@ -1060,33 +1193,29 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
         g.n4 = n4;
         g.n1 = n1;
         gather_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(g, n);
-        for (int a = 0; a < n4; ++a)
-            SPH_TRY(cudaMemcpyAsync(arr4[a], c.tmp4[a], (size_t)n * 16, cudaMemcpyDeviceToDevice, st));
-        for (int a = 0; a < n1; ++a)
-            SPH_TRY(cudaMemcpyAsync(arr1[a], c.tmp1[a], (size_t)n * 4, cudaMemcpyDeviceToDevice, st));
-        SPH_TRY(cudaMemcpyAsync(s.perm, c.tmp_perm, (size_t)n * 4, cudaMemcpyDeviceToDevice, st));
+        copy_back_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(g, n);
     }
     // recorded leaf ranges refer to the previous tree: mark them invalid
     SPH_TRY(cudaMemsetAsync(t.rec_ctl + 1, 0xff, sizeof(int), st));
     // 5. chop: tree (n_leaf) and groups (n_group)
-    chop_flags_kernel<<<grid_for(c, n, kCfTile), 256, 0, st>>>(s.keys, inst, n, p.n_leaf, p.n_group,
-                                                                t.lv_tree, t.lv_grp);
+    if (n < kCfTile * c.num_sms)
+        chop_flags_kernel<kCfSmall><<<grid_for(c, n, kCfSmall), 256, 0, st>>>(s.keys, inst, n, p.n_leaf,
+                                                                               p.n_group, t.lv_tree, t.lv_grp);
+    else
+        chop_flags_kernel<kCfTile><<<grid_for(c, n, kCfTile), 256, 0, st>>>(s.keys, inst, n, p.n_leaf,
+                                                                            p.n_group, t.lv_tree, t.lv_grp);
     // groups
-    int *gidx = (int *)c.tmp1[1];  // scratch: tmp1[1..] are free once copied back
-    SPH_TRY(scan_mode(c, t.lv_grp, gidx, n, 1, c.d_sizes + SZ_GROUPS, st));
-    group_write_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(t.lv_grp, gidx, n, t);
-    group_bounds_kernel<<<grid_for(c, n, 128), 128, 0, st>>>(pos, s.h, n, t, c.d_sizes, 0, nullptr);
+    SPH_TRY(scan_mode(c, t.lv_grp, nullptr, n, 1, c.d_sizes + SZ_GROUPS, st, t.grp_ref));
     // nodes
     int nb = div_up(n, kChopBlock);
     int *blk_off = (int *)c.tmp1[2];
     int *ntotal = c.d_sizes + 2;
     chop_count_kernel<<<nb, 256, 0, st>>>(t.lv_tree, n, t.blk_cnt, nb);
     SPH_TRY(scan_mode(c, t.blk_cnt, blk_off, kLevels * nb, 0, ntotal, st));
-    chop_write_kernel<<<nb, 256, 0, st>>>(t.lv_tree, n, blk_off, nb, t, c.d_err);
-    level_start_kernel<<<1, 32, 0, st>>>(blk_off, nb, ntotal, t, c.d_sizes);
-    node_finish_kernel<<<grid_for(c, t.cap_nodes, 256), 256, 0, st>>>(s.keys, inst, n, p.n_leaf, t,
-                                                                       c.d_sizes);
-    node_bounds_kernel<<<grid_for(c, t.cap_nodes, 128), 128, 0, st>>>(pos, s.h, t, c.d_sizes, 0, nullptr);
+    chop_write_kernel<<<nb, 256, 0, st>>>(t.lv_tree, n, blk_off, nb, ntotal, t, c.d_sizes, c.d_err);
+    node_finish_kernel<<<grid_for(c, node_cap_for(t, n), 256), 256, 0, st>>>(s.keys, inst, n, p.n_leaf, blk_off,
+                                                                              nb, t, c.d_sizes);
+    SPH_TRY(launch_bounds(c, s, 0, nullptr, st));
     return cudaGetLastError();
 }
 
@@ -1110,12 +1239,7 @@ cudaError_t update_hmax(Ctx &c, const sph_state &s, const sph_params &p, cudaStr
                         const int *gate)
 {
     (void)p;
-    Tree &t = c.tree;
-    node_bounds_kernel<<<grid_for(c, t.cap_nodes, 128), 128, 0, st>>>((const float4 *)s.pos, s.h, t,
-                                                                       c.d_sizes, 1, gate);
-    group_bounds_kernel<<<grid_for(c, s.n, 128), 128, 0, st>>>((const float4 *)s.pos, s.h,
-                                                               (int)s.n, t, c.d_sizes, 1, gate);
-    return cudaGetLastError();
+    return launch_bounds(c, s, 1, gate, st);
 }
 
 // Test hook for the bounded look-back: one block of a sort pass that takes
