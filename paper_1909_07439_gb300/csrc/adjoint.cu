@@ -8,10 +8,11 @@
 // its own equations and from its neighbours' equations.  No atomics, so the
 // results are deterministic.
 //
-// Force backward: the vector-Jacobian product of the pair term T_ij (the
-// contribution of j to a_i and du_i/dt, Eqs. 9-15 as the force pass computes
-// them) is a hand-written reverse sweep (force_pair_vjp), one sweep per pair
-// and side, in FP32 only (this GPU's FP64 rate is a small fraction of FP32's).
+// Force backward: the two terms of a pair that depend on a target k's inputs,
+// T_kj (the contribution of j to a_k and du_k/dt, Eqs. 9-15 as the force pass
+// computes them) and T_jk, are differentiated together by one hand-written
+// reverse sweep (force_pair_vjp): they share all their forward values.  FP32
+// only (this GPU's FP64 rate is a small fraction of FP32's).
 //
 // Density backward (implicit-function theorem): h_i solves
 // g_i = sum_j m_j W(r_ij, h_i) - M_i / h_i^3 = 0, M_i = m_i hfact^3, with
@@ -21,6 +22,8 @@
 //
 // The pair operations are templates on the smoothing kernel K (SphKernel<K>:
 // f, f', f'' and the support radius R).
+#include <algorithm>
+
 #include "kernels.cuh"
 #include "walk.cuh"
 
@@ -56,7 +59,7 @@ struct PairWalkSmem {
     int ej[kPW_TB][CAP];
 };
 
-// Op: struct with  Acc;  init(i, Acc&);  pair(i, j, Acc&);  reduce(Acc&, L);  store(i, Acc&)
+// Op: struct with  Acc;  init(i, Acc&);  pair(j, x_j and m_j, Acc&);  reduce(Acc&, L);  store(i, Acc&)
 template <int CAP, class Op>
 __global__ void __launch_bounds__(128) pairwalk_kernel(PairWalkArgs a, Op op)
 {
@@ -93,7 +96,7 @@ __global__ void __launch_bounds__(128) pairwalk_kernel(PairWalkArgs a, Op op)
             auto flush = [&]() {
                 if (act) {
                     const int len = sm.tlen[t];
-                    for (int e = sub; e < len; e += L) op.pair(i, sm.ej[t][e], acc);
+                    for (int e = sub; e < len; e += L) op.pair(sm.ej[t][e], __ldg(&a.pos[sm.ej[t][e]]), acc);
                 }
                 __syncwarp();
                 if (lane < nt) sm.tlen[lane] = 0;
@@ -148,12 +151,14 @@ __global__ void __launch_bounds__(128) pairwalk_kernel(PairWalkArgs a, Op op)
                     const int *__restrict__ lst = a.nl_idx + (size_t)i * a.nl_stride;
                     const float4 tp = sm.tp[t];
                     const float ht = sm.th[t];
+                    int jn = sub < len ? __ldcs(lst + sub) : 0;  // an entry ahead
                     for (int e = sub; e < len; e += L) {
-                        const int j = __ldcs(lst + e);
+                        const int j = jn;
+                        if (e + L < len) jn = __ldcs(lst + e + L);
                         const float4 pj = __ldg(&a.pos[j]);
                         const float r2 = canon_r2p(tp.x, tp.y, tp.z, pj.x, pj.y, pj.z, a.tree.per);
                         const float R = a.dens_set ? a.kr * ht : a.kr * fmaxf(ht, __ldg(&a.h[j]));
-                        if (r2 < R * R && (a.dens_set || j != i)) op.pair(i, j, acc);
+                        if (r2 < R * R && (a.dens_set || j != i)) op.pair(j, pj, acc);
                     }
                 }
                 __syncwarp();
@@ -172,11 +177,6 @@ __global__ void __launch_bounds__(128) pairwalk_kernel(PairWalkArgs a, Op op)
 }
 
 // ------------------------------------------------------------ force backward
-// Inputs of one particle in a pair term.
-struct PairIn {
-    float x[3], v[3], u, h, rho, om;
-};
-
 // P_i - P_j = (gamma - 1)(rho_i u_i - rho_j u_j) without FP64 (whose rate is
 // a small fraction of FP32's on this GPU): each product's rounding error is
 // recovered exactly with an FMA, and when the pressures are close the
@@ -194,179 +194,141 @@ __device__ __forceinline__ float pressure_diff(float gm1, float ri, float ui, fl
 // sqrt(x) for x >= 0 through the hardware reciprocal square root (0 at 0)
 __device__ __forceinline__ float fast_sqrt(float x) { return x > 0.f ? x * rsqrtf(x) : 0.f; }
 
-// Reverse-mode derivative of the pair term T_ij (particle I in the role of
-// i, J in the role of j, the same operations as the force pass): given the
-// cotangent w of (a_i xyz, du_i/dt), adds w . dT_ij / d(inputs of I) to g
-// and w . dT_ij / d alpha to *galpha (WANT_I), or w . dT_ij / d(inputs of J)
-// to g (otherwise).  r = 0 gives no term, the viscous terms act for vr < 0
-// only, |x| has derivative +1 at 0, and sqrt has derivative 0 at 0 (at equal
-// pressures the conduction term carries u_i - u_j times a zero speed).
-// Quotients and roots use the hardware approximations (a few ulp).
-template <bool WANT_I, int K>
-__device__ __forceinline__ void force_pair_vjp(const PairIn &I, const PairIn &J, float mj, float alpha,
-                                               float beta, float alpha_u, float gamma, float4 w,
-                                               const Period &P, PairIn &g, float &galpha)
+// A particle in a pair term: position and mass, velocity and u, (h, rho,
+// A = 1 / (rho Omega), c), the cotangent w of (a xyz, du/dt).
+struct PairIn {
+    float4 x, v, q, w;
+};
+
+// What a target's pairs add up to: the cotangents of x, v, u, h, rho and of
+// A and c (turned into those of rho, Omega and u once at the end), and twice
+// that of alpha_AV.
+struct PairGrad {
+    float x[3], v[3], u, h, rho, A, c, al;
+};
+
+// Reverse-mode derivative, with respect to the inputs of the target k, of
+//   S = w_k . T_kj + w_j . T_jk
+//     = -coef (W . d) / r + e_k E_k + e_j E_j + (e_k - e_j) alpha_u / 2 vsu (u_k - u_j) AF,
+// W = m_j w_k - m_k w_j (its acceleration part), e_k = m_j w_k.w, e_j = m_k w_j.w,
+// d = x_k - x_j, coef = sum of A p F over both, E = A ((gamma - 1) u vr F - D),
+// D = vsig vr^2 F / 2 for vr < 0, AF = sum of A F (the same operations as the
+// force pass).  r = 0 gives no term, the viscous terms act for vr < 0 only, and
+// sqrt has derivative 0 at 0 (at equal pressures the conduction term carries
+// u_k - u_j times a zero speed).  Quotients and roots use the hardware
+// approximations (a few ulp).  hk = 1 / h_k.  (One sweep over each of the two
+// terms by itself forms every forward value twice: 64^3 lattice 575 -> 427 us.)
+template <int K>
+__device__ __forceinline__ void force_pair_vjp(const PairIn &I, const PairIn &J, float hk, float alpha,
+                                               float beta, float alpha_u, float gm1, const Period &P,
+                                               PairGrad &g)
 {
-    const float gm1 = gamma - 1.f;
     // nearest images on the periodic axes (the wrap's derivative is 1)
-    const float dx = wrap_sep(I.x[0] - J.x[0], P.x), dy = wrap_sep(I.x[1] - J.x[1], P.y),
-                dz = wrap_sep(I.x[2] - J.x[2], P.z);
+    const float dx = wrap_sep(I.x.x - J.x.x, P.x), dy = wrap_sep(I.x.y - J.x.y, P.y),
+                dz = wrap_sep(I.x.z - J.x.z, P.z);
     const float r2 = dx * dx + dy * dy + dz * dz;
     if (!(r2 > 0.f)) return;
     const float rinv = rsqrtf(r2);
     const float r = r2 * rinv;
     // ---- forward values
-    const float hiinv = __fdividef(1.f, I.h), hjinv = __fdividef(1.f, J.h);
-    const float qi = r * hiinv, qj = r * hjinv;
-    const float dfi = SphKernel<K>::df(qi), dfj = SphKernel<K>::df(qj);
-    const float h2i = hiinv * hiinv, h2j = hjinv * hjinv;
-    const float Ki = SphKernel<K>::C * h2i * h2i, Kj = SphKernel<K>::C * h2j * h2j;  // C / h^4
-    const float Fi = dfi * Ki, Fj = dfj * Kj;
-    const float dvx = I.v[0] - J.v[0], dvy = I.v[1] - J.v[1], dvz = I.v[2] - J.v[2];
+    const float hj = __fdividef(1.f, J.q.x);
+    const float qk = r * hk, qj = r * hj;
+    const float h2k = hk * hk, h2j = hj * hj;
+    const float Kk = SphKernel<K>::C * h2k * h2k, Kj = SphKernel<K>::C * h2j * h2j;  // C / h^4
+    const float Fk = SphKernel<K>::df(qk) * Kk, Fj = SphKernel<K>::df(qj) * Kj;
+    const float dvx = I.v.x - J.v.x, dvy = I.v.y - J.v.y, dvz = I.v.z - J.v.z;
     const float sd = dvx * dx + dvy * dy + dvz * dz;
-    const float vr = sd * rinv;
+    const float vr = sd * rinv, vr2 = vr * vr;
     const float avr = fabsf(vr);
-    const float ci = fast_sqrt(gamma * gm1 * I.u), cj = fast_sqrt(gamma * gm1 * J.u);
-    const float vsi = alpha * ci + beta * avr;
     const bool visc = vr < 0.f;
-    const float vsj = alpha * cj + beta * avr;
-    const float avi = visc ? -0.5f * (vsi * vr) : 0.f;
-    const float avj = visc ? -0.5f * (vsj * vr) : 0.f;
-    const float duav = visc ? 0.5f * (vsi * vr * vr * Fi) : 0.f;
-    const float rhoinv_i = __fdividef(1.f, I.rho), rhoinv_j = __fdividef(1.f, J.rho);
-    const float Ai = rhoinv_i * __fdividef(1.f, I.om), Aj = rhoinv_j * __fdividef(1.f, J.om);
-    const float pi_ = gm1 * I.u + avi, pj_ = gm1 * J.u + avj;
-    const float Ti = Ai * pi_ * Fi, Tj = Aj * pj_ * Fj;
-    const float coef = mj * (Ti + Tj);
-    const float PD = pressure_diff(gm1, I.rho, I.u, J.rho, J.u);
-    const float APD = fabsf(PD);
-    const float Sinv = __fdividef(2.f, I.rho + J.rho);   // 1 / (rho_i + rho_j) / 2
-    const float X = APD * Sinv;
+    const float vsk = alpha * I.q.w + beta * avr, vsj = alpha * J.q.w + beta * avr;
+    const float Ak = I.q.z, Aj = J.q.z;
+    const float prk = gm1 * I.v.w, prj = gm1 * J.v.w;  // P / rho
+    const float pk = prk + (visc ? -0.5f * (vsk * vr) : 0.f), pj = prj + (visc ? -0.5f * (vsj * vr) : 0.f);
+    const float Dk = visc ? 0.5f * (vsk * vr2 * Fk) : 0.f;
+    const float coef = Ak * pk * Fk + Aj * pj * Fj;
+    const float PD = pressure_diff(gm1, I.q.y, I.v.w, J.q.y, J.v.w);
+    const float Sinv = __fdividef(2.f, I.q.y + J.q.y);   // 1 / ((rho_k + rho_j) / 2)
+    const float X = fabsf(PD) * Sinv;
     const float vsu = fast_sqrt(X);
-    const float du = I.u - J.u;
-    const float AF = Fi * Ai + Fj * Aj;
+    const float du = I.v.w - J.v.w;
+    const float AF = Fk * Ak + Fj * Aj;
     // ---- reverse sweep
-    float bui = 0.f, bhi = 0.f, brhoi = 0.f, bomi = 0.f;
-    float buj = 0.f, bhj = 0.f, brhoj = 0.f, bomj = 0.f;
-    float bal = 0.f;
-    // out_a = -coef rinv d
-    const float Wd = w.x * dx + w.y * dy + w.z * dz;
-    const float bcr = -Wd;
-    const float cri = -coef * rinv;
-    float bdx = cri * w.x, bdy = cri * w.y, bdz = cri * w.z;
-    float brinv = bcr * coef;
-    const float bcoef = bcr * rinv;
-    // out_u = mj E, E = gm1 u_i A_i vr F_i - A_i duav + 0.5 alpha_u vsu (u_i - u_j) AF
-    const float bE = w.w * mj;
-    const float hau = 0.5f * alpha_u * bE;
-    bui += bE * gm1 * Ai * vr * Fi + hau * vsu * AF;
-    buj += -hau * vsu * AF;
-    float bAi = bE * (gm1 * I.u * vr * Fi - duav);
-    float bvr = bE * gm1 * I.u * Ai * Fi;
-    float bFi = bE * gm1 * I.u * Ai * vr;
-    const float bduav = -bE * Ai;
-    const float bvsu = hau * du * AF;
-    const float bAF = hau * vsu * du;
-    // AF = F_i A_i + F_j A_j
-    bFi += bAF * Ai;
-    bAi += bAF * Fi;
-    float bFj = bAF * Aj;
-    float bAj = bAF * Fj;
-    // vsu = sqrt(|PD| / Srho), Srho = (rho_i + rho_j) / 2
+    const float mj = J.x.w, mk = I.x.w;
+    const float Wx = mj * I.w.x - mk * J.w.x, Wy = mj * I.w.y - mk * J.w.y, Wz = mj * I.w.z - mk * J.w.z;
+    const float ek = mj * I.w.w, ej = mk * J.w.w;
+    const float Wd = Wx * dx + Wy * dy + Wz * dz;
+    // -coef (W . d) rinv
+    const float cr = -coef * rinv;
+    float bdx = cr * Wx, bdy = cr * Wy, bdz = cr * Wz;
+    float brinv = -coef * Wd;
+    const float bcoef = -rinv * Wd;
+    // conduction
+    const float hau = 0.5f * alpha_u * (ek - ej);
+    float bu = hau * vsu * AF + ek * gm1 * Ak * vr * Fk;
+    const float bvsu = hau * du * AF, bAF = hau * vsu * du;
+    // pressure work and viscous heating
+    const float ekA = ek * Ak, ejA = ej * Aj;
+    float bA = ek * (prk * vr * Fk - Dk) + bAF * Fk;
+    float bvr = ekA * prk * Fk + ejA * prj * Fj;
+    float bFk = ekA * prk * vr + bAF * Ak;
+    float bFj = ejA * prj * vr + bAF * Aj;
+    // vsu = sqrt(|PD| / Srho), Srho = (rho_k + rho_j) / 2
     const float bX = vsu > 0.f ? __fdividef(0.5f * bvsu, vsu) : 0.f;
     const float bAPD = bX * Sinv;
-    const float bSrho = -bX * X * Sinv;
     const float bPD = PD < 0.f ? -bAPD : bAPD;
-    brhoi += bPD * gm1 * I.u + 0.5f * bSrho;
-    bui += bPD * gm1 * I.rho;
-    brhoj += -bPD * gm1 * J.u + 0.5f * bSrho;
-    buj += -bPD * gm1 * J.rho;
-    // coef = mj (T_i + T_j), T = A p F
-    const float bT = bcoef * mj;
-    bAi += bT * pi_ * Fi;
-    bFi += bT * Ai * pi_;
-    const float bpi = bT * Ai * Fi;
-    bAj += bT * pj_ * Fj;
-    bFj += bT * Aj * pj_;
-    const float bpj = bT * Aj * Fj;
-    bui += bpi * gm1;
-    buj += bpj * gm1;
-    float bavr = 0.f, bci = 0.f, bcj = 0.f;
+    g.rho += bPD * prk - 0.5f * bAPD * X;
+    bu += bPD * gm1 * I.q.y;
+    // coef = sum of A p F
+    bA += bcoef * pk * Fk;
+    bFk += bcoef * Ak * pk;
+    bFj += bcoef * Aj * pj;
+    const float bpk = bcoef * Ak * Fk, bpj = bcoef * Aj * Fj;
+    bu += bpk * gm1;
     if (visc) {
-        // avi = -vsi vr / 2, avj = -vsj vr / 2, duav = vsi vr^2 F_i / 2
-        const float bvsi = bpi * (-0.5f * vr) + bduav * 0.5f * vr * vr * Fi;
-        const float bvsj = bpj * (-0.5f * vr);
-        bvr += bpi * (-0.5f * vsi) + bpj * (-0.5f * vsj) + bduav * vsi * vr * Fi;
-        bFi += bduav * 0.5f * vsi * vr * vr;
-        bal += bvsi * ci + bvsj * cj;
-        bci += bvsi * alpha;
-        bcj += bvsj * alpha;
-        bavr += (bvsi + bvsj) * beta;
+        // p = (gamma - 1) u - vsig vr / 2, D = vsig vr^2 F / 2 with cotangents -ekA, -ejA
+        const float hvr = -0.5f * vr, hv2 = 0.5f * vr2;
+        const float bvsk = bpk * hvr - ekA * hv2 * Fk, bvsj = bpj * hvr - ejA * hv2 * Fj;
+        bvr += -0.5f * (bpk * vsk + bpj * vsj) - vr * (ekA * vsk * Fk + ejA * vsj * Fj);
+        bFk -= ekA * hv2 * vsk;
+        bFj -= ejA * hv2 * vsj;
+        g.al += bvsk * I.q.w + bvsj * J.q.w;
+        g.c += bvsk * alpha;
+        bvr -= (bvsk + bvsj) * beta;  // |vr| = -vr here
     }
-    // A = 1 / (rho Omega)
-    brhoi += -bAi * Ai * rhoinv_i;
-    bomi += -bAi * Ai * __fdividef(1.f, I.om);
-    brhoj += -bAj * Aj * rhoinv_j;
-    bomj += -bAj * Aj * __fdividef(1.f, J.om);
-    // c = sqrt(gamma gm1 u)
-    bui += ci > 0.f ? __fdividef(bci * gamma * gm1 * 0.5f, ci) : 0.f;
-    buj += cj > 0.f ? __fdividef(bcj * gamma * gm1 * 0.5f, cj) : 0.f;
-    // avr = |vr| (derivative +1 at 0)
-    bvr += vr < 0.f ? -bavr : bavr;
+    g.u += bu;
+    g.A += bA;
     // vr = sd rinv
     const float bsd = bvr * rinv;
     brinv += bvr * sd;
-    bdx += bsd * dvx;
-    bdy += bsd * dvy;
-    bdz += bsd * dvz;
     // F = C f'(q) / h^4, q = r / h
-    float br = 0.f;
-    {
-        const float bq = bFi * Ki * SphKernel<K>::d2f(qi);
-        bhi += -4.f * bFi * Fi * hiinv - bq * qi * hiinv;
-        br += bq * hiinv;
-    }
-    {
-        const float bq = bFj * Kj * SphKernel<K>::d2f(qj);
-        bhj += -4.f * bFj * Fj * hjinv - bq * qj * hjinv;
-        br += bq * hjinv;
-    }
+    const float bqk = bFk * Kk * SphKernel<K>::d2f(qk), bqj = bFj * Kj * SphKernel<K>::d2f(qj);
+    g.h -= hk * (4.f * bFk * Fk + bqk * qk);
     // rinv = 1 / r, r = |d|
-    br += -brinv * rinv * rinv;
-    bdx += br * rinv * dx;
-    bdy += br * rinv * dy;
-    bdz += br * rinv * dz;
-    if (WANT_I) {
-        g.x[0] += bdx;
-        g.x[1] += bdy;
-        g.x[2] += bdz;
-        g.v[0] += bsd * dx;
-        g.v[1] += bsd * dy;
-        g.v[2] += bsd * dz;
-        g.u += bui;
-        g.h += bhi;
-        g.rho += brhoi;
-        g.om += bomi;
-        galpha += bal;
-    } else {
-        // d = x_i - x_j, dv = v_i - v_j
-        g.x[0] -= bdx;
-        g.x[1] -= bdy;
-        g.x[2] -= bdz;
-        g.v[0] -= bsd * dx;
-        g.v[1] -= bsd * dy;
-        g.v[2] -= bsd * dz;
-        g.u += buj;
-        g.h += bhj;
-        g.rho += brhoj;
-        g.om += bomj;
+    const float br = (bqk * hk + bqj * hj - brinv * rinv * rinv) * rinv;
+    g.x[0] += bdx + bsd * dvx + br * dx;
+    g.x[1] += bdy + bsd * dvy + br * dy;
+    g.x[2] += bdz + bsd * dvz + br * dz;
+    g.v[0] += bsd * dx;
+    g.v[1] += bsd * dy;
+    g.v[2] += bsd * dz;
+}
+
+// (h, rho, 1 / (rho Omega), c) of every particle, as the force pass has it
+__global__ void bwd_prep_kernel(const float4 *__restrict__ vel, const float *__restrict__ h,
+                                const float *__restrict__ rho, const float *__restrict__ omega, int n,
+                                float gamma, float4 *__restrict__ prop)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const float c2 = gamma * (gamma - 1.f) * vel[i].w;
+        prop[i] = make_float4(h[i], rho[i], 1.f / (rho[i] * omega[i]), sqrtf(fmaxf(c2, 0.f)));
     }
 }
 
 template <int KER>
 struct ForceBwdOp {
-    const float4 *pos, *vel, *gacc;  // gacc: (dL/da xyz, dL/d(du/dt))
-    const float *h, *rho, *omega;
+    const float4 *pos, *vel, *prop, *gacc;  // gacc: (dL/da xyz, dL/d(du/dt))
+    const float *omega;
     float4 *gpos, *gvel;             // out: dL/dx (xyz, 0), dL/dv (xyz), dL/du (w)
     float *gh, *grho, *gom;          // out
     double *galpha;                  // out: accumulated (one atomic per target)
@@ -374,33 +336,21 @@ struct ForceBwdOp {
     Period per;
     struct Acc {
         PairIn K;     // the target's own inputs, loaded once
-        float mk;
-        float4 wk;    // the target's cotangent
-        PairIn g;
-        float ga;
+        float hk;
+        PairGrad g;
     };
-    __device__ PairIn load(int k) const
-    {
-        const float4 p = pos[k], v = vel[k];
-        return PairIn{{p.x, p.y, p.z}, {v.x, v.y, v.z}, v.w, h[k], rho[k], omega[k]};
-    }
     __device__ void init(int k, Acc &c) const
     {
-        c.K = load(k);
-        c.mk = pos[k].w;
-        c.wk = gacc[k];
-        c.g = PairIn{{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, 0.f, 0.f, 0.f, 0.f};
-        c.ga = 0.f;
+        c.K = PairIn{pos[k], vel[k], prop[k], gacc[k]};
+        c.hk = 1.f / c.K.q.x;
+        c.g = PairGrad{{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     }
     // the terms that land on k's inputs: from k's own equations (T_kj with
     // cotangent gacc[k]) and from j's (T_jk with cotangent gacc[j])
-    __device__ void pair(int k, int j, Acc &c) const
+    __device__ void pair(int j, float4 pj, Acc &c) const
     {
-        (void)k;
-        const PairIn J = load(j);
-        force_pair_vjp<true, KER>(c.K, J, pos[j].w, alpha, beta, alpha_u, gamma, c.wk, per, c.g, c.ga);
-        float unused = 0.f;
-        force_pair_vjp<false, KER>(J, c.K, c.mk, alpha, beta, alpha_u, gamma, gacc[j], per, c.g, unused);
+        const PairIn J{pj, __ldg(&vel[j]), __ldg(&prop[j]), __ldg(&gacc[j])};
+        force_pair_vjp<KER>(c.K, J, c.hk, alpha, beta, alpha_u, gamma - 1.f, per, c.g);
     }
     __device__ void reduce(Acc &c, int L) const
     {
@@ -413,18 +363,23 @@ struct ForceBwdOp {
             c.g.u += __shfl_xor_sync(0xffffffffu, c.g.u, o);
             c.g.h += __shfl_xor_sync(0xffffffffu, c.g.h, o);
             c.g.rho += __shfl_xor_sync(0xffffffffu, c.g.rho, o);
-            c.g.om += __shfl_xor_sync(0xffffffffu, c.g.om, o);
-            c.ga += __shfl_xor_sync(0xffffffffu, c.ga, o);
+            c.g.A += __shfl_xor_sync(0xffffffffu, c.g.A, o);
+            c.g.c += __shfl_xor_sync(0xffffffffu, c.g.c, o);
+            c.g.al += __shfl_xor_sync(0xffffffffu, c.g.al, o);
         }
     }
     __device__ void store(int k, Acc &c) const
     {
+        // A = 1 / (rho Omega), c = sqrt(gamma (gamma - 1) u)
+        const float bA = c.g.A * c.K.q.z, cs = c.K.q.w;
+        const float bu = cs > 0.f ? c.g.c * gamma * (gamma - 1.f) * 0.5f / cs : 0.f;
         gpos[k] = make_float4(c.g.x[0], c.g.x[1], c.g.x[2], 0.f);
-        gvel[k] = make_float4(c.g.v[0], c.g.v[1], c.g.v[2], c.g.u);
+        gvel[k] = make_float4(c.g.v[0], c.g.v[1], c.g.v[2], c.g.u + bu);
         gh[k] = c.g.h;
-        grho[k] = c.g.rho;
-        gom[k] = c.g.om;
-        atomicAdd(galpha, (double)c.ga);
+        grho[k] = c.g.rho - bA / c.K.q.y;
+        gom[k] = -bA / omega[k];
+        // T_kj counts here and in the sum of j
+        atomicAdd(galpha, 0.5 * (double)c.g.al);
     }
 };
 
@@ -444,24 +399,26 @@ struct DensBwd1Op {
     const float4 *pos;
     const float *h, *rho, *omega;
     const float *gh, *grho, *gom;  // cotangents of h, rho, Omega
-    float2 *coef;                  // out: (lambda, w)
+    float4 *coef;                  // out: (lambda, w, 1 / h, -)
     float hf3;
     Period per;
-    struct Acc { float S, S2; };
-    __device__ void init(int, Acc &c) const { c.S = 0.f; c.S2 = 0.f; }
-    __device__ void pair(int i, int j, Acc &c) const
+    struct Acc { float4 x; float hinv, S, S2; };
+    __device__ void init(int i, Acc &c) const
     {
-        float4 pi = pos[i], pj = pos[j];
-        float dx = wrap_sep(pi.x - pj.x, per.x), dy = wrap_sep(pi.y - pj.y, per.y),
-              dz = wrap_sep(pi.z - pj.z, per.z);
-        float r = fast_sqrt(dx * dx + dy * dy + dz * dz);
-        float hi = h[i], hinv = __fdividef(1.f, hi);
-        float q = r * hinv, f, df, d2f;
+        c.x = pos[i];
+        c.hinv = __fdividef(1.f, h[i]);
+        c.S = c.S2 = 0.f;
+    }
+    // sums without their factors C / h^4 and C / h^5
+    __device__ void pair(int, float4 pj, Acc &c) const
+    {
+        const float dx = wrap_sep(c.x.x - pj.x, per.x), dy = wrap_sep(c.x.y - pj.y, per.y),
+                    dz = wrap_sep(c.x.z - pj.z, per.z);
+        const float q = fast_sqrt(dx * dx + dy * dy + dz * dz) * c.hinv;
+        float f, df, d2f;
         kernel_all<K>(q, f, df, d2f);
-        float h4 = hinv * hinv * hinv * hinv;
-        constexpr float C = SphKernel<K>::C;
-        c.S += pj.w * (-C * (3.f * f + q * df) * h4);
-        c.S2 += pj.w * (C * (12.f * f + 8.f * q * df + q * q * d2f) * h4 * hinv);
+        c.S -= pj.w * (3.f * f + q * df);
+        c.S2 += pj.w * (12.f * f + 8.f * q * df + q * q * d2f);
     }
     __device__ void reduce(Acc &c, int L) const
     {
@@ -472,12 +429,13 @@ struct DensBwd1Op {
     }
     __device__ void store(int i, Acc &c) const
     {
-        float hi = h[i], M = pos[i].w * hf3;
-        float h3 = hi * hi * hi, h4 = h3 * hi;
-        float domdh = (4.f * h3 * c.S + h4 * c.S2) / (3.f * M);
-        float htot = gh[i] - 3.f * rho[i] / hi * grho[i] + gom[i] * domdh;
-        float lambda = htot * hi / (3.f * rho[i] * omega[i]);
-        coef[i] = make_float2(lambda, gom[i] * h4 / (3.f * M));
+        const float hi = h[i], M = c.x.w * hf3, hinv = 1.f / hi;
+        const float h4 = hi * hi * hi * hi;
+        // h^3 S and h^4 S2 of the full sums are C / h times these
+        const float domdh = SphKernel<K>::C * hinv * (4.f * c.S + c.S2) / (3.f * M);
+        const float htot = gh[i] - 3.f * rho[i] / hi * grho[i] + gom[i] * domdh;
+        const float lambda = htot * hi / (3.f * rho[i] * omega[i]);
+        coef[i] = make_float4(lambda, gom[i] * h4 / (3.f * M), hinv, 0.f);
     }
 };
 
@@ -485,33 +443,30 @@ struct DensBwd1Op {
 // c_ij = -lambda_i m_j F(r, h_i) + w_i m_j d2W/dh dr(r, h_i)
 template <int K>
 struct DensBwd2Op {
-    const float4 *pos;
-    const float *h;
-    const float2 *coef;
+    const float4 *pos, *coef;
     float4 *gpos;  // accumulated (+=)
     Period per;
-    struct Acc { float g[3]; };
-    __device__ void init(int, Acc &c) const { c.g[0] = c.g[1] = c.g[2] = 0.f; }
-    __device__ static float cterm(float r, float hh, float lam, float w, float m)
+    struct Acc { float4 x, q; float g[3]; };
+    __device__ void init(int k, Acc &c) const
     {
-        float hinv = __fdividef(1.f, hh), q = r * hinv, f, df, d2f;
-        kernel_all<K>(q, f, df, d2f);
-        float h4 = hinv * hinv * hinv * hinv;
-        constexpr float C = SphKernel<K>::C;
-        float F = C * df * h4;
-        float Whr = -C * (4.f * df + q * d2f) * h4 * hinv;
-        return m * (-lam * F + w * Whr);
+        c.x = pos[k];
+        c.q = coef[k];
+        c.g[0] = c.g[1] = c.g[2] = 0.f;
     }
-    __device__ void pair(int k, int j, Acc &c) const
+    __device__ static float cterm(float r, float4 q, float m)  // q = (lambda, w, 1 / h)
     {
-        float4 pk = pos[k], pj = pos[j];
-        float dx = wrap_sep(pk.x - pj.x, per.x), dy = wrap_sep(pk.y - pj.y, per.y),
-              dz = wrap_sep(pk.z - pj.z, per.z);
-        float r2 = dx * dx + dy * dy + dz * dz;
+        const float x = r * q.z, h2 = q.z * q.z;
+        const float df = SphKernel<K>::df(x), d2f = SphKernel<K>::d2f(x);
+        return -m * SphKernel<K>::C * h2 * h2 * (q.x * df + q.y * q.z * (4.f * df + x * d2f));
+    }
+    __device__ void pair(int j, float4 pj, Acc &c) const
+    {
+        const float dx = wrap_sep(c.x.x - pj.x, per.x), dy = wrap_sep(c.x.y - pj.y, per.y),
+                    dz = wrap_sep(c.x.z - pj.z, per.z);
+        const float r2 = dx * dx + dy * dy + dz * dz;
         if (!(r2 > 0.f)) return;
-        float rinv = rsqrtf(r2), r = r2 * rinv;
-        float2 ck = coef[k], cj = coef[j];
-        float s = (cterm(r, h[k], ck.x, ck.y, pj.w) + cterm(r, h[j], cj.x, cj.y, pk.w)) * rinv;
+        const float rinv = rsqrtf(r2), r = r2 * rinv;
+        const float s = (cterm(r, c.q, pj.w) + cterm(r, __ldg(&coef[j]), c.x.w)) * rinv;
         c.g[0] += s * dx;
         c.g[1] += s * dy;
         c.g[2] += s * dz;
@@ -581,9 +536,8 @@ static cudaError_t force_bwd_k(Ctx &c, const sph_state &s, const sph_params &p, 
     ForceBwdOp<K> op;
     op.pos = (const float4 *)s.pos;
     op.vel = (const float4 *)s.vel;
+    op.prop = c.prop;
     op.gacc = gacc;
-    op.h = s.h;
-    op.rho = s.rho;
     op.omega = s.omega;
     op.gpos = gpos;
     op.gvel = gvel;
@@ -600,6 +554,8 @@ static cudaError_t force_bwd_k(Ctx &c, const sph_state &s, const sph_params &p, 
     cudaError_t e = check_list_kernel(c, p, st);
     if (e == cudaSuccess) e = update_hmax(c, s, p, st);
     if (e != cudaSuccess) return e;
+    const int n = (int)s.n, grid = std::min(div_up(n, 256), c.num_sms * 16);
+    bwd_prep_kernel<<<grid, 256, 0, st>>>(op.vel, s.h, s.rho, s.omega, n, p.gamma, c.prop);
     return launch_pairwalk<96>(c, s, false, SphKernel<K>::R, op.per, op, st, nullptr);
 }
 
@@ -614,7 +570,7 @@ cudaError_t force_bwd(Ctx &c, const sph_state &s, const sph_params &p, const flo
 
 template <int K>
 static cudaError_t density_bwd_k(Ctx &c, const sph_state &s, const sph_params &p, const float *gh,
-                                 const float *grho, const float *gom, float4 *gpos, float2 *coef,
+                                 const float *grho, const float *gom, float4 *gpos, float4 *coef,
                                  cudaStream_t st, bool refresh_hmax)
 {
     DensBwd1Op<K> op1;
@@ -637,7 +593,6 @@ static cudaError_t density_bwd_k(Ctx &c, const sph_state &s, const sph_params &p
     if (e != cudaSuccess) return e;
     DensBwd2Op<K> op2;
     op2.pos = (const float4 *)s.pos;
-    op2.h = s.h;
     op2.coef = coef;
     op2.gpos = gpos;
     op2.per = op1.per;
@@ -645,7 +600,7 @@ static cudaError_t density_bwd_k(Ctx &c, const sph_state &s, const sph_params &p
 }
 
 cudaError_t density_bwd(Ctx &c, const sph_state &s, const sph_params &p, const float *gh,
-                        const float *grho, const float *gom, float4 *gpos, float2 *coef,
+                        const float *grho, const float *gom, float4 *gpos, float4 *coef,
                         cudaStream_t st, bool refresh_hmax)
 {
     if (p.kernel == 1) return density_bwd_k<1>(c, s, p, gh, grho, gom, gpos, coef, st, refresh_hmax);

@@ -31,7 +31,7 @@ cudaError_t force_bwd(Ctx &c, const sph_state &s, const sph_params &p, const flo
                       float4 *gpos, float4 *gvel, float *gh, float *grho, float *gom,
                       double *galpha, cudaStream_t st);
 cudaError_t density_bwd(Ctx &c, const sph_state &s, const sph_params &p, const float *gh,
-                        const float *grho, const float *gom, float4 *gpos, float2 *coef,
+                        const float *grho, const float *gom, float4 *gpos, float4 *coef,
                         cudaStream_t st, bool refresh_hmax = true);
 
 static int grid_r(const Ctx &c, int64_t n)
@@ -197,7 +197,7 @@ struct RolloutBuf {
     float4 *gx = nullptr, *gv = nullptr, *ga = nullptr;
     float4 *gacc_s = nullptr, *gpos_s = nullptr, *gvel_s = nullptr;
     float *gh_s = nullptr, *grho_s = nullptr, *gom_s = nullptr;
-    float2 *coef = nullptr;
+    float4 *coef = nullptr;
     unsigned char *flag = nullptr;
 };
 
@@ -274,7 +274,7 @@ cudaError_t ensure_rb(Ctx &c, int64_t n, int n_steps, int ck, RB **out)
     A(cudaMalloc((void **)&b.gh_s, N * 4));
     A(cudaMalloc((void **)&b.grho_s, N * 4));
     A(cudaMalloc((void **)&b.gom_s, N * 4));
-    A(cudaMalloc((void **)&b.coef, N * 8));
+    A(cudaMalloc((void **)&b.coef, N * 16));
     A(cudaMalloc((void **)&b.flag, N));
     if (e != cudaSuccess) {
         delete rb;
@@ -477,8 +477,8 @@ extern "C" sph_status sph_density_bwd(sph_ctx *h, const sph_state *s, const sph_
     if (!h || !s || !p || !d_gh || !d_grho || !d_gomega || !d_gpos) return SPH_ERR_INVALID_ARG;
     Ctx &c = h->impl;
     if (s->n < 1 || s->n > c.max_n || !adjoint_params_ok(p)) return SPH_ERR_INVALID_ARG;
-    // the per-particle multipliers use context scratch (one float2 per particle)
+    // the per-particle multipliers use context scratch (one float4 per particle)
     cudaError_t e = density_bwd(c, *s, *p, d_gh, d_grho, d_gomega, (float4 *)d_gpos,
-                                reinterpret_cast<float2 *>(c.tmp4[3]), (cudaStream_t)stream);
+                                c.tmp4[3], (cudaStream_t)stream);
     return e == cudaSuccess ? SPH_OK : SPH_ERR_CUDA;
 }
