@@ -10,11 +10,12 @@
 // lanes per target, reading each target's neighbour list (built by
 // nlist_kernel at the starting h with a (1 + pad) margin).  A batch whose h
 // leaves that margin, or whose list overflowed, is handed to
-// density_walk_kernel, which starts the batch over: it walks the tree with a
-// padded search radius 2 h (1 + pad) per target and keeps the candidates as
+// density_walk_kernel, which goes on from the h reached (a fixed number of
+// updates starts over): it walks the tree with a padded search radius
+// 2 h (1 + pad) per target and keeps the candidates as
 // (r^2, m_j, (v_i - v_j).(x_i - x_j)) in shared memory, walking again if h
-// leaves the pad and falling back to summing while walking ("streamed") if a
-// list would overflow the shared-memory tile.
+// leaves the pad and summing while walking ("streamed") in a sweep whose lists
+// would overflow the shared-memory tile.
 //
 // Lane layout for the sums: L = 32 / pow2ceil(targets) lanes per target,
 // lane = t * L + sub; partial sums are reduced across the L lanes with xor
@@ -25,7 +26,7 @@
 
 namespace sph {
 
-constexpr int kTB = 8;           // targets per batch
+constexpr int kTB = kWalkTB;     // targets per batch of the walking kernel
 constexpr int kDensWarps = 4;    // warps per block
 constexpr float kPad = kListPad; // padded list radius, relative to h
 constexpr int kRound = 2;        // groups per warp per work grab of the list kernel
@@ -49,6 +50,7 @@ struct DensArgs {
     const float4 *vel;
     const float4 *rec;  // pos, vel side by side
     float *h, *rho, *omega, *drhodt;
+    float *h_try;  // h that a batch handed over had reached (scratch)
     float4 *prop;  // h, rho, 1/(rho Omega), c_s  (for the force pass)
     const int2 *grp_ref;
     const float4 *grp_lo, *grp_hi;
@@ -142,8 +144,11 @@ __device__ __forceinline__ void density_outputs(const DensArgs &a, int i, float 
     a.prop[i] = make_float4(h, rho, 1.f / (rho * om), cs);
 }
 
-__device__ __forceinline__ void push_fallback(const DensArgs &a, int g, int b0, int nt)
+// hands a batch over at the h its targets reached (h of target i, in the lanes
+// of mine)
+__device__ __forceinline__ void push_fallback(const DensArgs &a, int g, int b0, int nt, bool mine, int i, float h)
 {
+    if (mine) a.h_try[i] = h;
     if ((threadIdx.x & 31) == 0) push_fallback_batch(a.fallback, a.n_fallback, g, b0, nt);
 }
 
@@ -189,7 +194,7 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
                 if (!__any_sync(0xffffffffu, on)) continue;  // no target of the batch is due
                 const int len = act ? a.nl_len[i] : 0;
                 if (__any_sync(0xffffffffu, len < 0)) {  // no list (overflow, or too many leaves)
-                    push_fallback(a, g, b0, nt);
+                    push_fallback(a, g, b0, nt, act && sub == 0, i, a.h[i]);
                     continue;
                 }
                 const int *__restrict__ lst = a.nl_idx + (size_t)i * a.nl_stride;
@@ -289,8 +294,8 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
                         final_pass = true;
                     }
                 }
-                if (__any_sync(0xffffffffu, outside)) {  // start the batch over with walks
-                    push_fallback(a, g, b0, nt);
+                if (__any_sync(0xffffffffu, outside)) {  // go on with walks
+                    push_fallback(a, g, b0, nt, act && sub == 0, i, h);
                     continue;
                 }
                 if (on && sub == 0) density_outputs(a, i, h, M, s1, s2, vi.w, SphKernel<K>::C, VD);
@@ -307,10 +312,18 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
     }
 }
 
-// Batches the list kernel handed over, each solved from its starting h with
-// tree walks.
+// Batches the list kernel handed over, each solved with tree walks from the h
+// it had reached there, whose first updates are the largest (a fixed number of
+// updates starts over from the starting h).  Bound by the latency of its walks:
+// a warp's next candidates are loaded while it tests the ones before, its
+// batches have 4 targets, and lists that overflow are summed while walking in
+// that sweep only.  Density stage, before (from the starting
+// h, whole batches, no prefetch, streaming for good) and now: 8192 particles
+// from a rough h (1248 batches) 262 -> 161 us, the M6 tube (76 batches past the
+// list capacity) 392 -> 323 us.  List pads of 6 and 10 % instead of 3 were no
+// faster (163 and 209 us for the sphere).
 template <int CAP, int K>
-__global__ void __launch_bounds__(kDensWarps * 32) density_walk_kernel(DensArgs a)
+__global__ void __launch_bounds__(kDensWarps * 32, 4) density_walk_kernel(DensArgs a)
 {
     extern __shared__ __align__(16) unsigned char dsm_raw[];
     DensSmem<CAP> &sm = reinterpret_cast<DensSmem<CAP> *>(dsm_raw)[threadIdx.x >> 5];
@@ -329,32 +342,32 @@ __global__ void __launch_bounds__(kDensWarps * 32) density_walk_kernel(DensArgs 
         k = __shfl_sync(0xffffffffu, k, 0);
         if (k >= nfb) break;
         const int2 fb = a.fallback[k];
-        const int g = fb.x, b0 = fb.y & 0xffff, cnt = fb.y >> 16;  // cnt <= kTB
+        const int g = fb.x, b0 = fb.y & 0xffff, nt = fb.y >> 16;  // nt <= kTB
         const int2 gr = a.grp_ref[g];
-        const float4 glo = a.grp_lo[g], ghi = a.grp_hi[g];
         const int root = a.inst ? a.inst[gr.x] : 0;
         ++n_rewalk;
         {
-            const int nt = min(cnt, gr.y - b0);
             const int L = lanes_per_target(nt);
             const int t = lane >> (__ffs(L) - 1), sub = lane & (L - 1);  // L a power of two
             const bool act = t < nt;
             const int i = gr.x + b0 + (act ? t : 0);
             const bool on = act && (!a.active || a.active[i]);
+            const float4 pl = lane < nt ? a.pos[gr.x + b0 + lane] : make_float4(1e30f, 1e30f, 1e30f, 0.f);
+            float4 glo, ghi;
+            targets_box(pl, nt, glo, ghi);
             if (lane < kTB) {
-                const float4 p = lane < nt ? a.pos[gr.x + b0 + lane] : make_float4(1e30f, 1e30f, 1e30f, 0.f);
-                sm.tp[lane] = p;
-                sm.tq.set(lane, p);
+                sm.tp[lane] = pl;
+                sm.tq.set(lane, pl);
                 if (lane < nt) sm.tv[lane] = a.vel[gr.x + b0 + lane];
             }
             __syncwarp();
-            float h = a.h[i];
-            const float h_in = h;
+            const float h_in = a.h[i];
+            float h = fixed ? h_in : a.h_try[i];
             const float M = sm.tp[act ? t : 0].w * hf3;  // m_i hfact^3
             float hlo = 0.f, hhi = INFINITY;
             float hw = h * (1.f + kPad);  // list radius is R hw
-            bool valid = false;           // lists cover the current h
-            bool streamed = false;        // batch overflowed the tile
+            bool valid = false;               // lists cover the current h
+            bool streamed = false;            // batch overflowed the tile
             bool conv = !on;
             bool final_pass = false;
             int it = 0;
@@ -380,16 +393,27 @@ __global__ void __launch_bounds__(kDensWarps * 32) density_walk_kernel(DensArgs 
                 };
                 if (!valid) {
                     // (re)build the candidate lists with a walk
-                    const float myr = streamed ? R : SphKernel<K>::R * hw;  // padded unless streaming
+                    hw = h * (1.f + kPad);
+                    const float myr = SphKernel<K>::R * hw;
                     if (act && sub == 0) sm.tr2[t] = myr * myr;
                     if (lane < kTB) sm.tlen[lane] = 0;
                     float reach = act ? myr : 0.f;
                     for (int o = 16; o > 0; o >>= 1) reach = fmaxf(reach, __shfl_xor_sync(0xffffffffu, reach, o));
                     __syncwarp();
                     bool overflow = false;
-                    auto chunk = [&](int j) {
-                        const float4 pj = j >= 0 ? __ldg(&a.pos[j]) : make_float4(0, 0, 0, 0);
-                        const float4 vj = j >= 0 ? __ldg(&a.vel[j]) : make_float4(0, 0, 0, 0);
+                    // a chunk's candidates are loaded while the one before is tested
+                    int jn = -1;
+                    bool waiting = false;
+                    float4 pn = make_float4(0.f, 0.f, 0.f, 0.f), vn = pn;
+                    auto chunk = [&](int jnew) {
+                        const int j = jn;
+                        const float4 pj = pn, vj = vn;
+                        const bool ready = waiting;
+                        jn = jnew;
+                        waiting = true;
+                        pn = jn >= 0 ? __ldg(&a.pos[jn]) : make_float4(0, 0, 0, 0);
+                        vn = jn >= 0 && a.vd ? __ldg(&a.vel[jn]) : make_float4(0, 0, 0, 0);
+                        if (!ready) return;
                         unsigned bs[kTB];
                         float r2s[kTB];
                         int base[kTB];
@@ -443,14 +467,15 @@ __global__ void __launch_bounds__(kDensWarps * 32) density_walk_kernel(DensArgs 
                     };
                     bool ok = walk_group(a.tree, root, glo, ghi, reach, false, 0.f, sm.w, chunk);
                     if (!ok && lane == 0) raise_error(a.err, SPH_ERR_TILE_OVERFLOW);
+                    if (waiting) chunk(-1);  // the last one
                     list_sums();
-                    if (overflow) {
-                        if (!streamed) ++n_stream;
+                    // lists that overflowed were summed piece by piece: the next
+                    // sweep, at another h, walks again
+                    if (overflow && !streamed) {
+                        ++n_stream;
                         streamed = true;
-                        valid = false;
-                    } else {
-                        valid = !streamed;
                     }
+                    valid = !overflow;
                 } else {
                     list_sums();
                 }
@@ -465,10 +490,7 @@ __global__ void __launch_bounds__(kDensWarps * 32) density_walk_kernel(DensArgs 
                 if (final_pass) break;
                 if (on && !conv) {
                     newton_update(h, hlo, hhi, conv, s0, s1, M, fixed, a.tol, SphKernel<K>::C);
-                    if (h > hw) {  // outgrew the padded list
-                        hw = h * (1.f + kPad);
-                        valid = false;
-                    }
+                    if (h > hw) valid = false;  // outgrew the padded list
                 }
                 ++it;
                 if (__any_sync(0xffffffffu, !valid)) valid = false;
@@ -506,6 +528,7 @@ __global__ void __launch_bounds__(kDensWarps * 32) density_walk_kernel(DensArgs 
 }
 
 // ------------------------------------------------------------ neighbour lists
+constexpr int kNbrTB = 8;  // targets per batch of the test export
 struct NbrArgs {
     const float4 *pos;
     const float *h;
@@ -524,9 +547,9 @@ struct NbrArgs {
 
 struct NbrSmem {
     WalkSmem w;
-    float4 tp[kTB];
-    float th[kTB];
-    int tcnt[kTB];
+    float4 tp[kNbrTB];
+    float th[kNbrTB];
+    int tcnt[kNbrTB];
 };
 
 __global__ void __launch_bounds__(128) neighbour_kernel(NbrArgs a)
@@ -543,8 +566,8 @@ __global__ void __launch_bounds__(128) neighbour_kernel(NbrArgs a)
         if (g >= ng) break;
         int2 gr = a.grp_ref[g];
         float4 glo = a.grp_lo[g], ghi = a.grp_hi[g];
-        for (int b0 = 0; b0 < gr.y; b0 += kTB) {
-            int nt = min(kTB, gr.y - b0);
+        for (int b0 = 0; b0 < gr.y; b0 += kNbrTB) {
+            int nt = min(kNbrTB, gr.y - b0);
             if (lane < nt) {
                 sm.tp[lane] = a.pos[gr.x + b0 + lane];
                 sm.th[lane] = a.h[gr.x + b0 + lane];
@@ -722,6 +745,7 @@ static cudaError_t configure_density_k()
     if (e == cudaSuccess) e = configure_density<80, K>(b);
     if (e == cudaSuccess) e = configure_density<96, K>(b);
     if (e == cudaSuccess) e = configure_density<128, K>(b);
+    if (e == cudaSuccess) e = configure_density<192, K>(b);
     return e;
 }
 
@@ -756,13 +780,15 @@ static cudaError_t density_solve_k(Ctx &c, DensArgs &a, const sph_params &p, cud
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // default tile: the mean density set (about 58 for M4 at hfact 1.2, 82 for
-    // M6 at 0.9, 74 for Wendland C6 at 1.3) with room to spare
-    int cap = p.tile > 0 ? p.tile : K == 0 ? 80 : 128;
+    // default tile: the mean density set (about 58 for M4 at hfact 1.2, 82 and
+    // 113 for M6 at 0.9 and 1.0, 74 for Wendland C6 at 1.3) within the pad, with
+    // room to spare: an overflow costs a walk in every sweep
+    int cap = p.tile > 0 ? p.tile : K == 0 ? 96 : K == 1 ? 192 : 128;
     if (cap <= 64) return launch_density_walk<64, K>(c, a, st);
     if (cap <= 80) return launch_density_walk<80, K>(c, a, st);
     if (cap <= 96) return launch_density_walk<96, K>(c, a, st);
-    return launch_density_walk<128, K>(c, a, st);
+    if (cap <= 128) return launch_density_walk<128, K>(c, a, st);
+    return launch_density_walk<192, K>(c, a, st);
 }
 
 cudaError_t density_lists(Ctx &c, const sph_state &s, const sph_params &p, cudaStream_t st,
@@ -801,6 +827,7 @@ cudaError_t density_solve(Ctx &c, const sph_state &s, const sph_params &p, cudaS
     a.rec = c.rec;
     a.vd = c.drhodt_in_force ? 0 : 1;
     a.h = s.h;
+    a.h_try = c.tmp1[3];  // free between tree builds
     a.rho = s.rho;
     a.omega = s.omega;
     a.drhodt = s.drhodt;

@@ -404,14 +404,36 @@ __device__ __forceinline__ int walk_leaves_wide(const WalkTree &T, int root, flo
     return ok && nout <= cap ? nout : -1;
 }
 
+// box of the nt targets at p (one per lane, lanes 0..nt-1)
+__device__ __forceinline__ void targets_box(float4 p, int nt, float4 &lo, float4 &hi)
+{
+    const int lane = threadIdx.x & 31;
+    lo = lane < nt ? p : make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+    hi = lane < nt ? p : make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
+    for (int o = 16; o > 0; o >>= 1) {
+        lo.x = fminf(lo.x, __shfl_xor_sync(0xffffffffu, lo.x, o));
+        lo.y = fminf(lo.y, __shfl_xor_sync(0xffffffffu, lo.y, o));
+        lo.z = fminf(lo.z, __shfl_xor_sync(0xffffffffu, lo.z, o));
+        hi.x = fmaxf(hi.x, __shfl_xor_sync(0xffffffffu, hi.x, o));
+        hi.y = fmaxf(hi.y, __shfl_xor_sync(0xffffffffu, hi.y, o));
+        hi.z = fmaxf(hi.z, __shfl_xor_sync(0xffffffffu, hi.z, o));
+    }
+}
+
 // Hand a batch of cnt targets of group g, from its target b0 on, to the
-// walking kernels, in items of at most 8 targets (their batch size):
-// item = (g, first target | count << 16).  Called by one lane.
+// walking kernels, in items of at most kWalkTB targets (their batch size):
+// item = (g, first target | count << 16).  Called by one lane.  A walk is a
+// serial chain, whose length grows with the targets that each of its candidates
+// is tested against: in batches of 4 instead of 8 the differentiable evaluation
+// of 30 k particles spends 650 instead of 947 us in its two density passes.
+// The size is fixed, so that an instance's sums do not depend on how many other
+// batches were handed over.
+constexpr int kWalkTB = 4;
 __device__ __forceinline__ void push_fallback_batch(int2 *fallback, int *n_fallback, int g, int b0,
                                                     int cnt)
 {
-    for (int k = 0; k < cnt; k += 8)
-        fallback[atomicAdd(n_fallback, 1)] = make_int2(g, (b0 + k) | (min(8, cnt - k) << 16));
+    for (int k = 0; k < cnt; k += kWalkTB)
+        fallback[atomicAdd(n_fallback, 1)] = make_int2(g, (b0 + k) | (min(kWalkTB, cnt - k) << 16));
 }
 
 // Candidate slots of a group: runs[m] = (first particle, first slot) for
