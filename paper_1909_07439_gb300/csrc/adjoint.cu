@@ -63,6 +63,7 @@ struct PairWalkSmem {
 template <int CAP, class Op>
 __global__ void __launch_bounds__(128) pairwalk_kernel(PairWalkArgs a, Op op)
 {
+    pdl_sync();
     extern __shared__ __align__(16) unsigned char pw_raw[];
     PairWalkSmem<CAP> &sm = reinterpret_cast<PairWalkSmem<CAP> *>(pw_raw)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -319,6 +320,7 @@ __global__ void bwd_prep_kernel(const float4 *__restrict__ vel, const float *__r
                                 const float *__restrict__ rho, const float *__restrict__ omega, int n,
                                 float gamma, float4 *__restrict__ prop)
 {
+    pdl_sync();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float c2 = gamma * (gamma - 1.f) * vel[i].w;
         prop[i] = make_float4(h[i], rho[i], 1.f / (rho[i] * omega[i]), sqrtf(fmaxf(c2, 0.f)));
@@ -524,7 +526,7 @@ static cudaError_t launch_pairwalk(Ctx &c, const sph_state &s, bool dens_set, fl
     a.err = c.d_err;
     cudaError_t e = cudaMemsetAsync(a.work, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
-    pairwalk_kernel<CAP, Op><<<c.num_sms * blocks, 128, smem, st>>>(a, op);
+    launch(pairwalk_kernel<CAP, Op>, c.num_sms * blocks, 128, smem, st, a, op);
     return cudaGetLastError();
 }
 
@@ -555,7 +557,7 @@ static cudaError_t force_bwd_k(Ctx &c, const sph_state &s, const sph_params &p, 
     if (e == cudaSuccess) e = update_hmax(c, s, p, st);
     if (e != cudaSuccess) return e;
     const int n = (int)s.n, grid = std::min(div_up(n, 256), c.num_sms * 16);
-    bwd_prep_kernel<<<grid, 256, 0, st>>>(op.vel, s.h, s.rho, s.omega, n, p.gamma, c.prop);
+    launch(bwd_prep_kernel, grid, 256, 0, st, op.vel, s.h, s.rho, s.omega, n, p.gamma, c.prop);
     return launch_pairwalk<96>(c, s, false, SphKernel<K>::R, op.per, op, st, nullptr);
 }
 

@@ -160,6 +160,7 @@ __device__ __forceinline__ void push_fallback(const DensArgs &a, int g, int b0, 
 template <int NPER, int K, bool PER, bool VD>
 __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
 {
+    pdl_sync();
     const int lane = threadIdx.x & 31;
     const uint64_t keep = l2_keep_policy();
     const int ng = a.sizes[SZ_GROUPS];
@@ -325,6 +326,7 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
 template <int CAP, int K>
 __global__ void __launch_bounds__(kDensWarps * 32, 4) density_walk_kernel(DensArgs a)
 {
+    pdl_sync();
     extern __shared__ __align__(16) unsigned char dsm_raw[];
     DensSmem<CAP> &sm = reinterpret_cast<DensSmem<CAP> *>(dsm_raw)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -554,6 +556,7 @@ struct NbrSmem {
 
 __global__ void __launch_bounds__(128) neighbour_kernel(NbrArgs a)
 {
+    pdl_sync();
     __shared__ NbrSmem smv[4];
     NbrSmem &sm = smv[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -605,6 +608,7 @@ __global__ void __launch_bounds__(128) neighbour_kernel(NbrArgs a)
 
 __global__ void scan_i64_kernel(int64_t *off, int n)
 {
+    pdl_sync();
     // single block exclusive scan of counts (test-only path, not timed)
     __shared__ int64_t carry;
     if (threadIdx.x == 0) carry = 0;
@@ -639,6 +643,7 @@ __global__ void list_set_kernel(const float4 *__restrict__ pos, const float *__r
                                 int stride, int mode, float kr, Period per, int64_t *off,
                                 int32_t *out, int *missing)
 {
+    pdl_sync();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int l = len[i];
         if (l < 0) {
@@ -732,7 +737,7 @@ static cudaError_t launch_density_walk(Ctx &c, const DensArgs &a, cudaStream_t s
     cudaError_t e = configure_density<CAP, K>(blocks);
     if (e != cudaSuccess) return e;
     size_t smem = sizeof(DensSmem<CAP>) * kDensWarps;
-    density_walk_kernel<CAP, K><<<c.num_sms * blocks, kDensWarps * 32, smem, st>>>(a);
+    launch(density_walk_kernel<CAP, K>, c.num_sms * blocks, kDensWarps * 32, smem, st, a);
     return cudaGetLastError();
 }
 
@@ -768,15 +773,15 @@ static cudaError_t density_solve_k(Ctx &c, DensArgs &a, const sph_params &p, cud
     const dim3 grid(c.num_sms * bl[wl]), block(32 * ps.warps);
     const bool per = a.tree.per.any();
     if (a.vd) {
-        if (ps.unroll == 4 && per) density_list_kernel<4, K, true, true><<<grid, block, 0, st>>>(a);
-        else if (ps.unroll == 4) density_list_kernel<4, K, false, true><<<grid, block, 0, st>>>(a);
-        else if (per) density_list_kernel<2, K, true, true><<<grid, block, 0, st>>>(a);
-        else density_list_kernel<2, K, false, true><<<grid, block, 0, st>>>(a);
+        if (ps.unroll == 4 && per) launch(density_list_kernel<4, K, true, true>, grid, block, 0, st, a);
+        else if (ps.unroll == 4) launch(density_list_kernel<4, K, false, true>, grid, block, 0, st, a);
+        else if (per) launch(density_list_kernel<2, K, true, true>, grid, block, 0, st, a);
+        else launch(density_list_kernel<2, K, false, true>, grid, block, 0, st, a);
     } else {
-        if (ps.unroll == 4 && per) density_list_kernel<4, K, true, false><<<grid, block, 0, st>>>(a);
-        else if (ps.unroll == 4) density_list_kernel<4, K, false, false><<<grid, block, 0, st>>>(a);
-        else if (per) density_list_kernel<2, K, true, false><<<grid, block, 0, st>>>(a);
-        else density_list_kernel<2, K, false, false><<<grid, block, 0, st>>>(a);
+        if (ps.unroll == 4 && per) launch(density_list_kernel<4, K, true, false>, grid, block, 0, st, a);
+        else if (ps.unroll == 4) launch(density_list_kernel<4, K, false, false>, grid, block, 0, st, a);
+        else if (per) launch(density_list_kernel<2, K, true, false>, grid, block, 0, st, a);
+        else launch(density_list_kernel<2, K, false, false>, grid, block, 0, st, a);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -876,17 +881,17 @@ cudaError_t list_sets(Ctx &c, const sph_state &s, const sph_params &p, int mode,
     if (e != cudaSuccess) return e;
     const int grid = c.num_sms * 8;
     const float kr = kernel_support(p.kernel);
-    list_set_kernel<<<grid, 256, 0, st>>>((const float4 *)s.pos, s.h, c.nl_idx, c.nl_len, n,
+    launch(list_set_kernel, grid, 256, 0, st, (const float4 *)s.pos, s.h, c.nl_idx, c.nl_len, n,
                                           c.nl_stride, mode, kr, period_of(p),
                                           d_off, nullptr, missing);
-    scan_i64_kernel<<<1, 1024, 0, st>>>(d_off, n);
+    launch(scan_i64_kernel, 1, 1024, 0, st, d_off, n);
     e = cudaMemcpyAsync(h_total, d_off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c.h_pinned + 4, missing, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return e;
     *h_missing = c.h_pinned[4];
     if (d_idx && *h_total <= cap) {
-        list_set_kernel<<<grid, 256, 0, st>>>((const float4 *)s.pos, s.h, c.nl_idx, c.nl_len, n,
+        launch(list_set_kernel, grid, 256, 0, st, (const float4 *)s.pos, s.h, c.nl_idx, c.nl_len, n,
                                               c.nl_stride, mode,
                                               kr, period_of(p), d_off, d_idx, missing);
         e = cudaStreamSynchronize(st);
@@ -916,8 +921,8 @@ cudaError_t neighbour_lists(Ctx &c, const sph_state &s, const sph_params &p, int
     int grid = c.num_sms * 4;
     cudaError_t e = cudaMemsetAsync(a.work, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
-    neighbour_kernel<<<grid, 128, 0, st>>>(a);
-    scan_i64_kernel<<<1, 1024, 0, st>>>(d_off, (int)s.n);
+    launch(neighbour_kernel, grid, 128, 0, st, a);
+    launch(scan_i64_kernel, 1, 1024, 0, st, d_off, (int)s.n);
     e = cudaMemcpyAsync(h_total, d_off + s.n, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return e;
     e = cudaStreamSynchronize(st);
@@ -926,7 +931,7 @@ cudaError_t neighbour_lists(Ctx &c, const sph_state &s, const sph_params &p, int
         a.idx = d_idx;
         e = cudaMemsetAsync(a.work, 0, sizeof(int), st);
         if (e != cudaSuccess) return e;
-        neighbour_kernel<<<grid, 128, 0, st>>>(a);
+        launch(neighbour_kernel, grid, 128, 0, st, a);
         e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return e;
     }

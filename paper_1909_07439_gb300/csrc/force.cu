@@ -262,6 +262,7 @@ struct ForceSums {
 template <int NPER, int K, bool PER>
 __global__ void __launch_bounds__(256, 3) force_list_kernel(ForceArgs a)
 {
+    pdl_sync();
     const int lane = threadIdx.x & 31;
     const uint64_t keep = l2_keep_policy();
     const int ng = a.sizes[SZ_GROUPS];
@@ -359,6 +360,7 @@ __global__ void __launch_bounds__(256, 3) force_list_kernel(ForceArgs a)
 template <int CAP, int K>
 __global__ void __launch_bounds__(kForceWarps * 32) force_walk_kernel(ForceArgs a)
 {
+    pdl_sync();
     extern __shared__ __align__(16) unsigned char fsm_raw[];
     ForceSmem<CAP> &sm = reinterpret_cast<ForceSmem<CAP> *>(fsm_raw)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -491,6 +493,7 @@ __global__ void force_prep_kernel(const float4 *__restrict__ pos, const float4 *
                                   float4 *__restrict__ frec, int n, float gamma, float alpha, float kr,
                                   float gc, float h_lim, int *err)
 {
+    pdl_sync();
     bool bad = false, neg = false, wide = false;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float4 v = vel[i];
@@ -575,7 +578,7 @@ static cudaError_t launch_force_walk(Ctx &c, const ForceArgs &a, cudaStream_t st
     cudaError_t e = configure_force<CAP, K>(blocks);
     if (e != cudaSuccess) return e;
     size_t smem = sizeof(ForceSmem<CAP>) * kForceWarps;
-    force_walk_kernel<CAP, K><<<c.num_sms * blocks, kForceWarps * 32, smem, st>>>(a);
+    launch(force_walk_kernel<CAP, K>, c.num_sms * blocks, kForceWarps * 32, smem, st, a);
     return cudaGetLastError();
 }
 
@@ -602,7 +605,7 @@ cudaError_t force_prep(Ctx &c, const sph_state &s, const sph_params &p, cudaStre
     const int n = (int)s.n;
     int grid = (n + 255) / 256;
     if (grid > c.num_sms * 16) grid = c.num_sms * 16;
-    force_prep_kernel<<<grid, 256, 0, st>>>((const float4 *)s.pos, (const float4 *)s.vel, s.h, s.rho,
+    launch(force_prep_kernel, grid, 256, 0, st, (const float4 *)s.pos, (const float4 *)s.vel, s.h, s.rho,
                                             s.omega, c.prop, c.frec, n, p.gamma, p.alpha_av,
                                             kernel_support(p.kernel), kernel_gc(p.kernel),
                                             periodic_h_limit(p), c.d_err);
@@ -624,10 +627,10 @@ static cudaError_t force_launch_k(Ctx &c, ForceArgs &a, const sph_params &p, con
     const int u = ps.unroll == 4 ? 1 : 0, wl = ps.warps == 8 ? 3 : ps.warps == 4 ? 2 : ps.warps == 2 ? 1 : 0;
     const int grid = c.num_sms * bl[u][wl];
     const bool per = a.tree.per.any();
-    if (u && per) force_list_kernel<4, K, true><<<grid, 32 * ps.warps, 0, st>>>(a);
-    else if (u) force_list_kernel<4, K, false><<<grid, 32 * ps.warps, 0, st>>>(a);
-    else if (per) force_list_kernel<2, K, true><<<grid, 32 * ps.warps, 0, st>>>(a);
-    else force_list_kernel<2, K, false><<<grid, 32 * ps.warps, 0, st>>>(a);
+    if (u && per) launch(force_list_kernel<4, K, true>, grid, 32 * ps.warps, 0, st, a);
+    else if (u) launch(force_list_kernel<4, K, false>, grid, 32 * ps.warps, 0, st, a);
+    else if (per) launch(force_list_kernel<2, K, true>, grid, 32 * ps.warps, 0, st, a);
+    else launch(force_list_kernel<2, K, false>, grid, 32 * ps.warps, 0, st, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // the walking kernel needs node and group h_max of the final h; refreshed

@@ -73,6 +73,7 @@ struct GravArgs {
 __global__ void gravity_moments_kernel(const float4 *__restrict__ pos, Tree t, float4 *com, float4 *q0,
                                        float4 *q1, const int *sizes, float theta)
 {
+    pdl_sync();
     const int nn = sizes[SZ_NODES];
     auto finish = [&](int k, float M, float3 X, float Q[6]) {
         const float4 lo = t.node_lo[k], hi = t.node_hi[k];
@@ -146,6 +147,7 @@ __global__ void gravity_moments_kernel(const float4 *__restrict__ pos, Tree t, f
 
 __global__ void __launch_bounds__(kGWarps * 32) gravity_kernel(GravArgs a)
 {
+    pdl_sync();
     __shared__ GravSmem smv[kGWarps];
     GravSmem &sm = smv[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -404,7 +406,7 @@ cudaError_t gravity_pass(Ctx &c, const sph_state &s, const sph_params &p, float4
     const int n = (int)s.n;
     int mgrid = (int)((c.tree.cap_nodes + 255) / 256);
     if (mgrid > c.num_sms * 16) mgrid = c.num_sms * 16;
-    gravity_moments_kernel<<<mgrid, 256, 0, st>>>((const float4 *)s.pos, c.tree, c.g_com, c.g_q0, c.g_q1,
+    launch(gravity_moments_kernel, mgrid, 256, 0, st, (const float4 *)s.pos, c.tree, c.g_com, c.g_q0, c.g_q1,
                                                   c.d_sizes, p.grav_theta);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -429,7 +431,7 @@ cudaError_t gravity_pass(Ctx &c, const sph_state &s, const sph_params &p, float4
     (void)n;
     e = cudaMemsetAsync(a.work, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
-    gravity_kernel<<<c.num_sms * blocks, kGWarps * 32, 0, st>>>(a);
+    launch(gravity_kernel, c.num_sms * blocks, kGWarps * 32, 0, st, a);
     return cudaGetLastError();
 }
 

@@ -28,6 +28,7 @@ __global__ void kick_drift_kernel(const float4 *__restrict__ pos, const float4 *
                                   const float *d_dt, const int *__restrict__ inst, Period per,
                                   float3 plo)
 {
+    pdl_sync();
     auto wrap = [](float x, float L, float lo) {
         if (L > 0.f) {
             const float hi = lo + L;
@@ -58,6 +59,7 @@ __global__ void kick_close_kernel(float4 *__restrict__ vel, const float4 *__rest
                                   const float4 *__restrict__ vhalf, int n, const float *d_dt,
                                   double *d_time, int *err, const int *__restrict__ inst)
 {
+    pdl_sync();
     float dt = *d_dt, hdt = 0.5f * dt;
     bool neg = false;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -77,6 +79,7 @@ __global__ void kick_close_kernel(float4 *__restrict__ vel, const float4 *__rest
 // per-instance simulation time
 __global__ void time_batch_kernel(const float *d_dt, double *d_time, int n_inst)
 {
+    pdl_sync();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n_inst; k += gridDim.x * blockDim.x)
         d_time[k] += (double)d_dt[k];
 }
@@ -85,6 +88,7 @@ __global__ void time_batch_kernel(const float *d_dt, double *d_time, int n_inst)
 // when the warp lies inside one instance (positive floats order as ints)
 __global__ void dt_batch_init_kernel(int *dtmin, int n_inst)
 {
+    pdl_sync();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n_inst; k += gridDim.x * blockDim.x)
         dtmin[k] = 0x7f800000;  // +inf
 }
@@ -92,6 +96,7 @@ __global__ void dt_batch_init_kernel(int *dtmin, int n_inst)
 __global__ void dt_batch_kernel(const float *__restrict__ h, const float *__restrict__ vs,
                                 const int *__restrict__ inst, int n, int *dtmin)
 {
+    pdl_sync();
     for (int i0 = blockIdx.x * blockDim.x; i0 < n; i0 += gridDim.x * blockDim.x) {
         int i = i0 + threadIdx.x;
         bool in = i < n;
@@ -109,6 +114,7 @@ __global__ void dt_batch_kernel(const float *__restrict__ h, const float *__rest
 
 __global__ void dt_batch_final_kernel(const int *dtmin, int n_inst, float c_cour, float *d_dt)
 {
+    pdl_sync();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n_inst; k += gridDim.x * blockDim.x)
         d_dt[k] = c_cour * __int_as_float(dtmin[k]);
 }
@@ -118,6 +124,7 @@ __global__ void __launch_bounds__(256) dt_block_kernel(const float *__restrict__
                                                        const float *__restrict__ vs, int n,
                                                        float *blockmin)
 {
+    pdl_sync();
     __shared__ float sm[8];
     float m = INFINITY;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
@@ -134,6 +141,7 @@ __global__ void __launch_bounds__(256) dt_block_kernel(const float *__restrict__
 
 __global__ void dt_final_kernel(const float *blockmin, int nb, float c_cour, float *d_dt)
 {
+    pdl_sync();
     float m = INFINITY;
     for (int b = threadIdx.x; b < nb; b += 32) m = fminf(m, blockmin[b]);
     for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -146,6 +154,7 @@ __global__ void __launch_bounds__(256) conserved_block_kernel(const float4 *__re
                                                               const float4 *__restrict__ vel, int n,
                                                               double *part, int nb)
 {
+    pdl_sync();
     __shared__ double sm[8][256];
     double e[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -172,6 +181,7 @@ __global__ void __launch_bounds__(256) conserved_block_kernel(const float4 *__re
 
 __global__ void conserved_final_kernel(const double *part, int nb, double *out8)
 {
+    pdl_sync();
     int k = threadIdx.x;
     if (k < 8) {
         double s = 0.0;
@@ -209,6 +219,7 @@ __global__ void block_substep_kernel(float4 *__restrict__ pos, float4 *__restric
                                      int n, int j, int max_level, const float *d_dt_min, Period per,
                                      float3 plo, int *err)
 {
+    pdl_sync();
     bool any_bad = false;
     const float dtm = *d_dt_min;
     auto wrap = [](float x, float L, float lo) {
@@ -253,6 +264,7 @@ __global__ void block_close_kernel(float4 *__restrict__ vel, const float4 *__res
                                    const uint32_t *__restrict__ perm, const int *__restrict__ level,
                                    int n, int max_level, const float *d_dt_min, double *d_time, int *err)
 {
+    pdl_sync();
     const float dtm = *d_dt_min;
     bool neg = false;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -276,6 +288,7 @@ __global__ void block_levels_kernel(const float *__restrict__ h, const float *__
                                     const uint32_t *__restrict__ perm, int n, float c_cour,
                                     int max_level, const float *d_dt_min, int *level)
 {
+    pdl_sync();
     const float dtm = *d_dt_min;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float du = fabsf(acc[i].w);
@@ -291,7 +304,7 @@ cudaError_t block_substep(Ctx &c, const sph_state &s, const sph_params &p, const
                           int max_level, const float *d_dt_min, cudaStream_t st)
 {
     const int n = (int)s.n;
-    block_substep_kernel<<<grid_n(c, n, 256), 256, 0, st>>>(
+    launch(block_substep_kernel, grid_n(c, n, 256), 256, 0, st, 
         (float4 *)s.pos, (float4 *)s.vel, (const float4 *)s.acc, c.vhalf, c.active, s.perm,
         d_level, n, j, max_level, d_dt_min, period_of(p), box_lo_of(p), c.d_err);
     return cudaGetLastError();
@@ -301,7 +314,7 @@ cudaError_t block_close(Ctx &c, const sph_state &s, const int *d_level, int max_
                         const float *d_dt_min, double *d_time, cudaStream_t st)
 {
     const int n = (int)s.n;
-    block_close_kernel<<<grid_n(c, n, 256), 256, 0, st>>>((float4 *)s.vel, (const float4 *)s.acc,
+    launch(block_close_kernel, grid_n(c, n, 256), 256, 0, st, (float4 *)s.vel, (const float4 *)s.acc,
                                                           c.vhalf, c.active, s.perm, d_level, n,
                                                           max_level, d_dt_min, d_time, c.d_err);
     return cudaGetLastError();
@@ -311,7 +324,7 @@ cudaError_t block_levels(Ctx &c, const sph_state &s, const sph_params &p, int ma
                          const float *d_dt_min, int *d_level, cudaStream_t st)
 {
     const int n = (int)s.n;
-    block_levels_kernel<<<grid_n(c, n, 256), 256, 0, st>>>(s.h, s.vsigmax, (const float4 *)s.vel,
+    launch(block_levels_kernel, grid_n(c, n, 256), 256, 0, st, s.h, s.vsigmax, (const float4 *)s.vel,
                                                            (const float4 *)s.acc, s.perm, n, p.c_cour,
                                                            max_level, d_dt_min, d_level);
     return cudaGetLastError();
@@ -321,7 +334,7 @@ cudaError_t kick_drift(Ctx &c, const sph_state &s, const sph_params &p, const fl
                        cudaStream_t st, const Batch *batch)
 {
     int n = (int)s.n;
-    kick_drift_kernel<<<grid_n(c, n, 256), 256, 0, st>>>(
+    launch(kick_drift_kernel, grid_n(c, n, 256), 256, 0, st, 
         (const float4 *)s.pos, (const float4 *)s.vel, (const float4 *)s.acc, s.h, s.perm, c.tmp4[0],
         c.tmp4[1], c.tmp4[2], c.tmp1[0], c.tmp_perm, n, d_dt, batch ? c.inst : nullptr,
         period_of(p), box_lo_of(p));
@@ -332,11 +345,11 @@ cudaError_t kick_close(Ctx &c, const sph_state &s, const float *d_dt, double *d_
                        cudaStream_t st, const Batch *batch)
 {
     int n = (int)s.n;
-    kick_close_kernel<<<grid_n(c, n, 256), 256, 0, st>>>((float4 *)s.vel, (const float4 *)s.acc,
+    launch(kick_close_kernel, grid_n(c, n, 256), 256, 0, st, (float4 *)s.vel, (const float4 *)s.acc,
                                                          c.vhalf, n, d_dt, d_time, c.d_err,
                                                          batch ? c.inst : nullptr);
     if (batch && d_time)
-        time_batch_kernel<<<div_up(batch->n_inst, 256), 256, 0, st>>>(d_dt, d_time, batch->n_inst);
+        launch(time_batch_kernel, div_up(batch->n_inst, 256), 256, 0, st, d_dt, d_time, batch->n_inst);
     return cudaGetLastError();
 }
 
@@ -346,14 +359,14 @@ cudaError_t courant_dt(Ctx &c, const sph_state &s, const sph_params &p, float *d
     int n = (int)s.n;
     if (batch) {
         const int ni = batch->n_inst;
-        dt_batch_init_kernel<<<div_up(ni, 256), 256, 0, st>>>(c.dtmin_inst, ni);
-        dt_batch_kernel<<<grid_n(c, n, 256), 256, 0, st>>>(s.h, s.vsigmax, c.inst, n, c.dtmin_inst);
-        dt_batch_final_kernel<<<div_up(ni, 256), 256, 0, st>>>(c.dtmin_inst, ni, p.c_cour, d_dt);
+        launch(dt_batch_init_kernel, div_up(ni, 256), 256, 0, st, c.dtmin_inst, ni);
+        launch(dt_batch_kernel, grid_n(c, n, 256), 256, 0, st, s.h, s.vsigmax, c.inst, n, c.dtmin_inst);
+        launch(dt_batch_final_kernel, div_up(ni, 256), 256, 0, st, c.dtmin_inst, ni, p.c_cour, d_dt);
         return cudaGetLastError();
     }
     int nb = grid_n(c, n, 256);
-    dt_block_kernel<<<nb, 256, 0, st>>>(s.h, s.vsigmax, n, c.red_f);
-    dt_final_kernel<<<1, 32, 0, st>>>(c.red_f, nb, p.c_cour, d_dt);
+    launch(dt_block_kernel, nb, 256, 0, st, s.h, s.vsigmax, n, c.red_f);
+    launch(dt_final_kernel, 1, 32, 0, st, c.red_f, nb, p.c_cour, d_dt);
     return cudaGetLastError();
 }
 
@@ -361,9 +374,9 @@ cudaError_t conserved(Ctx &c, const sph_state &s, double *d_out8, cudaStream_t s
 {
     int n = (int)s.n;
     int nb = grid_n(c, n, 256);
-    conserved_block_kernel<<<nb, 256, 0, st>>>((const float4 *)s.pos, (const float4 *)s.vel, n,
+    launch(conserved_block_kernel, nb, 256, 0, st, (const float4 *)s.pos, (const float4 *)s.vel, n,
                                                c.red_d, nb);
-    conserved_final_kernel<<<1, 32, 0, st>>>(c.red_d, nb, d_out8);
+    launch(conserved_final_kernel, 1, 32, 0, st, c.red_d, nb, d_out8);
     return cudaGetLastError();
 }
 

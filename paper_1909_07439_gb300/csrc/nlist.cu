@@ -287,6 +287,7 @@ __device__ __forceinline__ int test_chunks(const NlistArgs &a, NlistSmem &sm, in
 template <bool PER, int CAP>
 __global__ void __launch_bounds__(kNlWarps * 32, 7) nlist_kernel(NlistArgs a)
 {
+    pdl_sync();
     __shared__ NlistSmem smv[kNlWarps];
     NlistSmem &sm = smv[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -480,11 +481,11 @@ static cudaError_t launch_nlist(Ctx &c, const NlistArgs &a, int blocks, cudaStre
     const dim3 grid(c.num_sms * blocks), block(kNlWarps * 32);
     const bool per = a.tree.per.any();
     if (a.cap == 128) {
-        if (per) nlist_kernel<true, 128><<<grid, block, 0, st>>>(a);
-        else nlist_kernel<false, 128><<<grid, block, 0, st>>>(a);
+        if (per) launch(nlist_kernel<true, 128>, grid, block, 0, st, a);
+        else launch(nlist_kernel<false, 128>, grid, block, 0, st, a);
     } else if (a.cap == 192) {
-        if (per) nlist_kernel<true, 192><<<grid, block, 0, st>>>(a);
-        else nlist_kernel<false, 192><<<grid, block, 0, st>>>(a);
+        if (per) launch(nlist_kernel<true, 192>, grid, block, 0, st, a);
+        else launch(nlist_kernel<false, 192>, grid, block, 0, st, a);
     } else {
         return cudaErrorInvalidValue;
     }

@@ -42,11 +42,13 @@ static int grid_r(const Ctx &c, int64_t n)
 
 __global__ void iota_kernel(uint32_t *p, int n)
 {
+    pdl_sync();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = i;
 }
 
 __global__ void probe_flag_kernel(const int64_t *probes, int np, int n, unsigned char *flag)
 {
+    pdl_sync();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < np; k += gridDim.x * blockDim.x) {
         int64_t p = probes[k];
         if (p >= 0 && p < n) flag[p] = 1;
@@ -57,6 +59,7 @@ __global__ void probe_flag_kernel(const int64_t *probes, int np, int n, unsigned
 __global__ void loss_block_kernel(const float *rho, const uint32_t *perm,
                                   const unsigned char *flag, int n, double *part)
 {
+    pdl_sync();
     __shared__ double sm[256];
     double s = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
@@ -72,6 +75,7 @@ __global__ void loss_block_kernel(const float *rho, const uint32_t *perm,
 
 __global__ void loss_final_kernel(const double *part, int nb, int np, double *loss)
 {
+    pdl_sync();
     if (threadIdx.x == 0) {
         double s = 0.0;
         for (int b = 0; b < nb; ++b) s += part[b];
@@ -84,6 +88,7 @@ __global__ void loss_final_kernel(const double *part, int nb, int np, double *lo
 __global__ void gather_cot_kernel(const uint32_t *perm, const float4 *ga, const float4 *gv,
                                   const float *dts, int k, int n, float4 *gacc_s)
 {
+    pdl_sync();
     const float hdt = 0.5f * dts[k];
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
         uint32_t o = perm[s];
@@ -96,6 +101,7 @@ __global__ void gather_cot_kernel(const uint32_t *perm, const float4 *ga, const 
 __global__ void loss_grho_kernel(const float *rho, const uint32_t *perm, const unsigned char *flag,
                                  int n, int np, float *grho)
 {
+    pdl_sync();
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x)
         if (flag[perm[s]]) grho[s] += 2.f * rho[s] / (float)np;
 }
@@ -106,6 +112,7 @@ __global__ void scatter_cot_kernel(const uint32_t *perm, const float4 *gpos_s, c
                                    const float *dts, int k, int n, float4 *gx, float4 *gv,
                                    float4 *ga)
 {
+    pdl_sync();
     const float dt = dts[k], hdt = 0.5f * dt;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
         uint32_t o = perm[s];
@@ -123,6 +130,7 @@ __global__ void scatter_cot_kernel(const uint32_t *perm, const float4 *gpos_s, c
 __global__ void final_grad_kernel(const uint32_t *perm, const float4 *gv, const float4 *gvel_s,
                                   int n, float *out)
 {
+    pdl_sync();
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
         uint32_t o = perm[s];
         float4 a = gv[o], b = gvel_s[s];
@@ -325,7 +333,7 @@ cudaError_t load_init(Ctx &c, sph_state &w, const sph_state &init, cudaStream_t 
     RT(cudaMemcpyAsync(w.vel, init.vel, n * 16, cudaMemcpyDeviceToDevice, st));
     RT(cudaMemcpyAsync(w.h, init.h, n * 4, cudaMemcpyDeviceToDevice, st));
     RT(cudaMemsetAsync(w.acc, 0, n * 16, st));
-    iota_kernel<<<grid_r(c, n), 256, 0, st>>>(w.perm, (int)n);
+    launch(iota_kernel, grid_r(c, n), 256, 0, st, w.perm, (int)n);
     return cudaGetLastError();
 }
 
@@ -355,9 +363,9 @@ cudaError_t rollout(Ctx &c, RolloutBuf &b, const sph_state &init, const sph_para
         }
     }
     RT(cudaMemsetAsync(b.flag, 0, n, st));
-    probe_flag_kernel<<<grid_r(c, np), 256, 0, st>>>(probes, np, n, b.flag);
-    loss_block_kernel<<<nb, 256, 0, st>>>(w.rho, w.perm, b.flag, n, b.part);
-    loss_final_kernel<<<1, 32, 0, st>>>(b.part, nb, np, b.d_loss);
+    launch(probe_flag_kernel, grid_r(c, np), 256, 0, st, probes, np, n, b.flag);
+    launch(loss_block_kernel, nb, 256, 0, st, w.rho, w.perm, b.flag, n, b.part);
+    launch(loss_final_kernel, 1, 32, 0, st, b.part, nb, np, b.d_loss);
     if (!grad) return cudaGetLastError();
     // ---- backward
     RT(cudaMemsetAsync(b.gx, 0, (size_t)n * 16, st));
@@ -383,21 +391,21 @@ cudaError_t rollout(Ctx &c, RolloutBuf &b, const sph_state &init, const sph_para
             // permutation is the identity) and its neighbour lists at the final h
             RT(build_tree(c, w, p, true, st));
             RT(density_lists(c, w, p, st, nullptr, false));
-            gather_cot_kernel<<<nb, 256, 0, st>>>(w.perm, b.ga, b.gv, b.dts, k, n, b.gacc_s);
+            launch(gather_cot_kernel, nb, 256, 0, st, w.perm, b.ga, b.gv, b.dts, k, n, b.gacc_s);
             RT(force_bwd(c, w, p, b.gacc_s, b.gpos_s, b.gvel_s, b.gh_s, b.grho_s, b.gom_s,
                          b.d_galpha, st));
             if (k == K - 1)
-                loss_grho_kernel<<<nb, 256, 0, st>>>(w.rho, w.perm, b.flag, n, np, b.grho_s);
+                launch(loss_grho_kernel, nb, 256, 0, st, w.rho, w.perm, b.flag, n, np, b.grho_s);
             // force_bwd refreshed node and group h_max for this h
             RT(density_bwd(c, w, p, b.gh_s, b.grho_s, b.gom_s, b.gpos_s, b.coef, st, false));
-            scatter_cot_kernel<<<nb, 256, 0, st>>>(w.perm, b.gpos_s, b.gvel_s, b.dts, k, n, b.gx,
+            launch(scatter_cot_kernel, nb, 256, 0, st, w.perm, b.gpos_s, b.gvel_s, b.dts, k, n, b.gx,
                                                    b.gv, b.ga);
         }
     }
     // ---- the initial force evaluation: (a0, du0) depend on v0, u0 and alpha
     RT(load_init(c, w, init, st));
     RT(evaluate(c, w, p, b.d_dt, st));
-    gather_cot_kernel<<<nb, 256, 0, st>>>(w.perm, b.ga, b.gv, b.dts, K, n, b.gacc_s);
+    launch(gather_cot_kernel, nb, 256, 0, st, w.perm, b.ga, b.gv, b.dts, K, n, b.gacc_s);
     return cudaGetLastError();
 }
 
@@ -446,7 +454,7 @@ extern "C" sph_status sph_rollout(sph_ctx *h, const sph_state *init, const sph_p
         e = force_bwd(c, w, *p, b.gacc_s, b.gpos_s, b.gvel_s, b.gh_s, b.grho_s, b.gom_s,
                       b.d_galpha, st);
         if (e != cudaSuccess) return SPH_ERR_CUDA;
-        final_grad_kernel<<<grid_r(c, n), 256, 0, st>>>(w.perm, b.gv, b.gvel_s, n, d_gvel);
+        launch(final_grad_kernel, grid_r(c, n), 256, 0, st, w.perm, b.gv, b.gvel_s, n, d_gvel);
         if (cudaMemcpyAsync(h_galpha, b.d_galpha, sizeof(double), cudaMemcpyDeviceToHost, st) !=
             cudaSuccess)
             return SPH_ERR_CUDA;

@@ -218,6 +218,34 @@ struct Period {
 inline Period period_of(const sph_params &p) { return Period{p.box_len[0], p.box_len[1], p.box_len[2]}; }
 inline float3 box_lo_of(const sph_params &p) { return make_float3(p.box_lo[0], p.box_lo[1], p.box_lo[2]); }
 
+// Every kernel of the passes is launched as a programmatic dependent of the
+// kernel before it on the stream and begins with pdl_sync(): its blocks are set
+// up while the last blocks of that kernel still run, wait there until it has
+// finished and its writes are visible, and then let the next kernel's blocks be
+// set up.  A step is some 40 short kernels that each depend on the one before:
+// PDLMEAS
+__device__ __forceinline__ void pdl_sync()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... P, class... A>
+inline cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---------------------------------------------------------------------------
 // launchers (host functions) implemented in the .cu files
 // ---------------------------------------------------------------------------

@@ -53,6 +53,7 @@ __device__ __forceinline__ uint64_t spread21(uint32_t v)
 // ------------------------------------------------------------ bbox + checks
 __global__ void bbox_init_kernel(int *bb)
 {
+    pdl_sync();
     if (threadIdx.x < 3) bb[threadIdx.x] = 0x7fffffff;           // min of ordered ints
     else if (threadIdx.x < 6) bb[threadIdx.x] = (int)0x80000000; // max
 }
@@ -60,6 +61,7 @@ __global__ void bbox_init_kernel(int *bb)
 __global__ void bbox_kernel(const float4 *__restrict__ pos, const float *__restrict__ h, int n,
                             int *bb, int *err)
 {
+    pdl_sync();
     int mn[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff};
     int mx[3] = {(int)0x80000000, (int)0x80000000, (int)0x80000000};
     bool bad = false;
@@ -98,6 +100,7 @@ __global__ void bbox_kernel(const float4 *__restrict__ pos, const float *__restr
 // batch: one box per instance (6 ordered ints each), warp-combined atomics
 __global__ void bbox_batch_init_kernel(int *bb, int n_inst)
 {
+    pdl_sync();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 6 * n_inst; k += gridDim.x * blockDim.x)
         bb[k] = (k % 6) < 3 ? 0x7fffffff : (int)0x80000000;
 }
@@ -105,6 +108,7 @@ __global__ void bbox_batch_init_kernel(int *bb, int n_inst)
 __global__ void bbox_batch_kernel(const float4 *__restrict__ pos, const float *__restrict__ h,
                                   const int *__restrict__ inst, int n, int *bb, int *err)
 {
+    pdl_sync();
     for (int i0 = blockIdx.x * blockDim.x; i0 < n; i0 += gridDim.x * blockDim.x) {
         int i = i0 + threadIdx.x;
         bool in = i < n;
@@ -154,6 +158,7 @@ __global__ void morton_kernel(const float4 *__restrict__ pos, const int *__restr
                               const int *bb, uint64_t *__restrict__ keys, uint32_t *__restrict__ idx,
                               Period per, float3 plo, int *err)
 {
+    pdl_sync();
     float lo[3], s;
     box_scale(bb, lo, s);
     const float L[3] = {per.x, per.y, per.z}, pl[3] = {plo.x, plo.y, plo.z};
@@ -233,6 +238,7 @@ __global__ void __launch_bounds__(256) rs_ghist_kernel(const uint64_t *__restric
                                                        const int *__restrict__ inst, int n,
                                                        uint32_t *ghist)
 {
+    pdl_sync();
     __shared__ uint32_t h[10][256];
     for (int k = threadIdx.x; k < 10 * 256; k += 256) (&h[0][0])[k] = 0;
     __syncthreads();
@@ -279,6 +285,7 @@ __global__ void __launch_bounds__(256) rs_ghist_kernel(const uint64_t *__restric
 // gstart[p][d] = exclusive scan of ghist[p][.]   (block p)
 __global__ void __launch_bounds__(256) rs_gscan_kernel(const uint32_t *ghist, uint32_t *gstart)
 {
+    pdl_sync();
     __shared__ uint32_t ws[8];
     uint32_t ex;
     block_scan_256(ghist[blockIdx.x * 256 + threadIdx.x], ex, ws);
@@ -296,6 +303,7 @@ __global__ void __launch_bounds__(RS_T, 4) rs_onesweep_kernel(
     const uint32_t *__restrict__ gstart, uint32_t *status, int *tile_counter, int *err,
     const int *gate, int spin_cap)
 {
+    pdl_sync();
     if (gate && *gate == 0) return;  // a pass of the full sort that is not needed
     __shared__ uint32_t gbase[256];   // first output slot of each digit for this tile
     __shared__ uint32_t tstart[256];  // first slot of each digit in the sorted tile
@@ -414,6 +422,7 @@ __global__ void __launch_bounds__(RS_T, 4) rs_onesweep_kernel(
 constexpr int kFixRun = 32;
 __global__ void rs_fixup_kernel(uint64_t *keys, uint32_t *vals, int n, int *full)
 {
+    pdl_sync();
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
         const uint64_t top = keys[s] >> 32;
         if (s > 0 && (keys[s - 1] >> 32) == top) continue;        // inside a run
@@ -454,6 +463,7 @@ __global__ void __launch_bounds__(kRankE * kRankP) rank_sort_kernel(const uint64
                                                                     uint64_t *__restrict__ kout,
                                                                     uint32_t *__restrict__ order)
 {
+    pdl_sync();
     __shared__ uint64_t sk[kRankTile];
     __shared__ int si[BATCH ? kRankTile : 1];
     const int part = threadIdx.x & (kRankP - 1);
@@ -505,6 +515,7 @@ struct GatherArgs {
 
 __global__ void gather_kernel(GatherArgs g, int n)
 {
+    pdl_sync();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         uint32_t o = g.order[k];
 #pragma unroll
@@ -526,6 +537,7 @@ __global__ void gather_kernel(GatherArgs g, int n)
 // the gathered arrays back into the state (one launch for all of them)
 __global__ void copy_back_kernel(GatherArgs g, int n)
 {
+    pdl_sync();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
 #pragma unroll
         for (int a = 0; a < 4; ++a)
@@ -549,6 +561,7 @@ __device__ __forceinline__ int scan_in(const int *in, int i, int n, int mode)
 
 __global__ void __launch_bounds__(SC_T) scan_reduce_kernel(const int *in, int n, int mode, int *part)
 {
+    pdl_sync();
     __shared__ uint32_t ws[8];
     int base = blockIdx.x * SC_CHUNK + threadIdx.x * SC_I;
     int s = 0;
@@ -561,6 +574,7 @@ __global__ void __launch_bounds__(SC_T) scan_reduce_kernel(const int *in, int n,
 
 __global__ void __launch_bounds__(SC_T) scan_part_kernel(int *part, int nb, int *total)
 {
+    pdl_sync();
     __shared__ uint32_t ws[8];
     uint32_t carry = 0;
     for (int b = 0; b < nb; b += SC_T) {
@@ -578,6 +592,7 @@ __global__ void __launch_bounds__(SC_T) scan_part_kernel(int *part, int nb, int 
 __global__ void __launch_bounds__(SC_T) scan_down_kernel(const int *in, int *out, int n, int mode,
                                                          const int *part, int2 *starts)
 {
+    pdl_sync();
     __shared__ uint32_t ws[8];
     int base = blockIdx.x * SC_CHUNK + threadIdx.x * SC_I;
     int v[SC_I], s = 0;
@@ -602,6 +617,7 @@ constexpr int SC1_T = 1024, kScanOne = SC1_T * SC_I;
 __global__ void __launch_bounds__(SC1_T) scan_one_kernel(const int *in, int *out, int n, int mode,
                                                          int *total, int2 *starts)
 {
+    pdl_sync();
     __shared__ int ws[32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int carry = 0;
@@ -642,14 +658,14 @@ static cudaError_t scan_mode(Ctx &c, const int *in, int *out, int n, int mode, i
                              cudaStream_t st, int2 *starts = nullptr)
 {
     if (n <= kScanOne) {
-        scan_one_kernel<<<1, SC1_T, 0, st>>>(in, out, n, mode, total_dev, starts);
+        launch(scan_one_kernel, 1, SC1_T, 0, st, in, out, n, mode, total_dev, starts);
         return cudaGetLastError();
     }
     int nb = div_up(n, SC_CHUNK);
     if (nb > c.scan_part_cap) return cudaErrorInvalidValue;
-    scan_reduce_kernel<<<nb, SC_T, 0, st>>>(in, n, mode, c.scan_part);
-    scan_part_kernel<<<1, SC_T, 0, st>>>(c.scan_part, nb, total_dev);
-    scan_down_kernel<<<nb, SC_T, 0, st>>>(in, out, n, mode, c.scan_part, starts);
+    launch(scan_reduce_kernel, nb, SC_T, 0, st, in, n, mode, c.scan_part);
+    launch(scan_part_kernel, 1, SC_T, 0, st, c.scan_part, nb, total_dev);
+    launch(scan_down_kernel, nb, SC_T, 0, st, in, out, n, mode, c.scan_part, starts);
     return cudaGetLastError();
 }
 
@@ -726,6 +742,7 @@ __global__ void __launch_bounds__(256) chop_flags_kernel(const uint64_t *__restr
                                                          int t_leaf, int t_group, int *lv_tree,
                                                          int *lv_grp)
 {
+    pdl_sync();
     // local index i <-> slot t0 - kCfHalo + i
     constexpr int R = TILE + 2 * kCfHalo;
     __shared__ signed char sb[R], sq[R], sm[R], s0[R], s1[R];
@@ -786,6 +803,7 @@ __device__ __forceinline__ int chop_warp_levels(const int *__restrict__ lv, int 
 __global__ void __launch_bounds__(256) chop_count_kernel(const int *__restrict__ lv, int n,
                                                          int *blk_cnt, int nb)
 {
+    pdl_sync();
     __shared__ int cnt[kLevels];
     if (threadIdx.x < kLevels) cnt[threadIdx.x] = 0;
     __syncthreads();
@@ -809,6 +827,7 @@ __global__ void __launch_bounds__(256) chop_write_kernel(const int *__restrict__
                                                          const int *__restrict__ blk_off, int nb,
                                                          const int *total, Tree t, int *sizes, int *err)
 {
+    pdl_sync();
     __shared__ int wcnt[kLevels][8];
     if (blockIdx.x == 0 && threadIdx.x == 0) sizes[SZ_NODES] = min(*total, t.cap_nodes);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -880,6 +899,7 @@ __global__ void node_finish_kernel(const uint64_t *__restrict__ keys, const int 
                                    int n, int T, const int *__restrict__ blk_off, int nb, Tree t,
                                    const int *sizes)
 {
+    pdl_sync();
     const int nn = sizes[SZ_NODES];
     // first node of level L (blk_off: the nodes per level and block, scanned)
     auto level_start = [&](int L) { return L < kLevels ? min(blk_off[L * nb], nn) : nn; };
@@ -1000,6 +1020,7 @@ __global__ void __launch_bounds__(128) bounds_kernel(const float4 *__restrict__ 
                                                      int n, Tree t, const int *sizes, int what, const int *gate,
                                                      int nb_nodes)
 {
+    pdl_sync();
     if (gate && *gate == 0) return;
     if ((int)blockIdx.x < nb_nodes) node_bounds(pos, h, t, sizes[SZ_NODES], what, blockIdx.x, nb_nodes);
     else group_bounds(pos, h, n, t, sizes[SZ_GROUPS], what, blockIdx.x - nb_nodes, gridDim.x - nb_nodes);
@@ -1010,6 +1031,7 @@ __global__ void __launch_bounds__(128) bounds_kernel(const float4 *__restrict__ 
 // offs[n_inst] = n (one block)
 __global__ void offsets_check_kernel(const int64_t *__restrict__ offs, int n_inst, int n, int *bad, int *err)
 {
+    pdl_sync();
     bool b = false;
     for (int k = threadIdx.x; k <= n_inst; k += blockDim.x)
         b |= k == 0 ? offs[0] != 0
@@ -1030,6 +1052,7 @@ __global__ void offsets_check_kernel(const int64_t *__restrict__ offs, int n_ins
 __global__ void instance_map_kernel(const int64_t *__restrict__ offs, int n_inst, int n, const int *bad,
                                     int *inst)
 {
+    pdl_sync();
     const bool valid = *bad == 0;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         if (!valid) {
@@ -1063,8 +1086,8 @@ static int grid_for(const Ctx &c, int64_t n, int block)
 cudaError_t instance_map(Ctx &c, const int64_t *d_offsets, int n_inst, int n, cudaStream_t st)
 {
     int *bad = c.d_sizes + SZ_BAD_OFFSETS;
-    offsets_check_kernel<<<1, 1024, 0, st>>>(d_offsets, n_inst, n, bad, c.d_err);
-    instance_map_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(d_offsets, n_inst, n, bad, c.inst);
+    launch(offsets_check_kernel, 1, 1024, 0, st, d_offsets, n_inst, n, bad, c.d_err);
+    launch(instance_map_kernel, grid_for(c, n, 256), 256, 0, st, d_offsets, n_inst, n, bad, c.inst);
     return cudaGetLastError();
 }
 
@@ -1074,7 +1097,7 @@ static int64_t node_cap_for(const Tree &t, int64_t n) { return std::min<int64_t>
 static cudaError_t launch_bounds(Ctx &c, const sph_state &s, int what, const int *gate, cudaStream_t st)
 {
     const int nb = grid_for(c, node_cap_for(c.tree, s.n), 128), gb = grid_for(c, s.n, 128);
-    bounds_kernel<<<nb + gb, 128, 0, st>>>((const float4 *)s.pos, s.h, (int)s.n, c.tree, c.d_sizes, what, gate, nb);
+    launch(bounds_kernel, nb + gb, 128, 0, st, (const float4 *)s.pos, s.h, (int)s.n, c.tree, c.d_sizes, what, gate, nb);
     return cudaGetLastError();
 }
 
@@ -1107,14 +1130,14 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
     const float *h_in = kicked ? c.tmp1[0] : s.h;
     // 1. bounding box (per instance in a batch) and input checks
     if (batch) {
-        bbox_batch_init_kernel<<<div_up(6 * batch->n_inst, 256), 256, 0, st>>>(bb, batch->n_inst);
-        bbox_batch_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(pos_in, h_in, inst, n, bb, c.d_err);
+        launch(bbox_batch_init_kernel, div_up(6 * batch->n_inst, 256), 256, 0, st, bb, batch->n_inst);
+        launch(bbox_batch_kernel, grid_for(c, n, 256), 256, 0, st, pos_in, h_in, inst, n, bb, c.d_err);
     } else {
-        bbox_init_kernel<<<1, 32, 0, st>>>(bb);
-        bbox_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(pos_in, h_in, n, bb, c.d_err);
+        launch(bbox_init_kernel, 1, 32, 0, st, bb);
+        launch(bbox_kernel, grid_for(c, n, 256), 256, 0, st, pos_in, h_in, n, bb, c.d_err);
     }
     // 2. keys
-    morton_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(pos_in, inst, n, bb, s.keys, c.idx_a,
+    launch(morton_kernel, grid_for(c, n, 256), 256, 0, st, pos_in, inst, n, bb, s.keys, c.idx_a,
                                                       period_of(p), box_lo_of(p), c.d_err);
     // 3. sort (key, slot): few particles by counting ranks, else the radix sort,
     //    where a batch adds stable passes on the instance id, which put every
@@ -1123,8 +1146,8 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
     uint32_t *vin = c.idx_a, *vout = c.idx_b;
     if (n <= kRankSort) {
         const int grid = div_up(n, kRankE);
-        if (batch) rank_sort_kernel<true><<<grid, kRankE * kRankP, 0, st>>>(kin, inst, n, kout, vout);
-        else rank_sort_kernel<false><<<grid, kRankE * kRankP, 0, st>>>(kin, nullptr, n, kout, vout);
+        if (batch) launch(rank_sort_kernel<true>, grid, kRankE * kRankP, 0, st, kin, inst, n, kout, vout);
+        else launch(rank_sort_kernel<false>, grid, kRankE * kRankP, 0, st, kin, nullptr, n, kout, vout);
         std::swap(kin, kout);
         std::swap(vin, vout);
     } else {
@@ -1137,13 +1160,13 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
         SPH_TRY(cudaMemsetAsync(c.rs_tiles, 0, sizeof(int) * (kRsSlots + 1), st));
         SPH_TRY(cudaMemsetAsync(c.rs_status, 0, sizeof(uint32_t) * 256 * (size_t)ntiles * nslot, st));
         const int gh_grid = (int)std::max<int64_t>(1, std::min<int64_t>(div_up(n, 256 * RS_GE), 4 * (int64_t)c.num_sms));
-        rs_ghist_kernel<<<gh_grid, 256, 0, st>>>(kin, inst, n, c.rs_ghist);
-        rs_gscan_kernel<<<ndigit, 256, 0, st>>>(c.rs_ghist, c.rs_gstart);
+        launch(rs_ghist_kernel, gh_grid, 256, 0, st, kin, inst, n, c.rs_ghist);
+        launch(rs_gscan_kernel, ndigit, 256, 0, st, c.rs_ghist, c.rs_gstart);
         int slot = 0;
         auto pass = [&](int digit, const int *gate) {
             const int *dinst = digit >= 8 ? inst : nullptr;
             const int shift = digit >= 8 ? 8 * (digit - 8) : 8 * digit;
-            rs_onesweep_kernel<<<ntiles, RS_T, 0, st>>>(kin, vin, kout, vout, dinst, n, shift,
+            launch(rs_onesweep_kernel, ntiles, RS_T, 0, st, kin, vin, kout, vout, dinst, n, shift,
                                                         c.rs_gstart + 256 * digit,
                                                         c.rs_status + (size_t)256 * ntiles * slot,
                                                         c.rs_tiles + slot, c.d_err, gate, RS_SPIN);
@@ -1152,7 +1175,7 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
             std::swap(vin, vout);  // the gated passes come in an even number
         };
         for (int digit = 4; digit < 8; ++digit) pass(digit, nullptr);
-        rs_fixup_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(kin, vin, n, full);
+        launch(rs_fixup_kernel, grid_for(c, n, 256), 256, 0, st, kin, vin, n, full);
         for (int digit = 0; digit < 8; ++digit) pass(digit, full);
         if (batch) {
             pass(8, nullptr);
@@ -1180,7 +1203,7 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
         g.tperm = s.perm;
         g.n4 = 3;
         g.n1 = 1;
-        gather_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(g, n);
+        launch(gather_kernel, grid_for(c, n, 256), 256, 0, st, g, n);
     } else {
         // gather into the temporaries, then copy back
         float4 *arr4[4] = {(float4 *)s.pos, (float4 *)s.vel, (float4 *)s.acc, nullptr};
@@ -1192,17 +1215,17 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
         g.tperm = c.tmp_perm;
         g.n4 = n4;
         g.n1 = n1;
-        gather_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(g, n);
-        copy_back_kernel<<<grid_for(c, n, 256), 256, 0, st>>>(g, n);
+        launch(gather_kernel, grid_for(c, n, 256), 256, 0, st, g, n);
+        launch(copy_back_kernel, grid_for(c, n, 256), 256, 0, st, g, n);
     }
     // recorded leaf ranges refer to the previous tree: mark them invalid
     SPH_TRY(cudaMemsetAsync(t.rec_ctl + 1, 0xff, sizeof(int), st));
     // 5. chop: tree (n_leaf) and groups (n_group)
     if (n < kCfTile * c.num_sms)
-        chop_flags_kernel<kCfSmall><<<grid_for(c, n, kCfSmall), 256, 0, st>>>(s.keys, inst, n, p.n_leaf,
+        launch(chop_flags_kernel<kCfSmall>, grid_for(c, n, kCfSmall), 256, 0, st, s.keys, inst, n, p.n_leaf,
                                                                                p.n_group, t.lv_tree, t.lv_grp);
     else
-        chop_flags_kernel<kCfTile><<<grid_for(c, n, kCfTile), 256, 0, st>>>(s.keys, inst, n, p.n_leaf,
+        launch(chop_flags_kernel<kCfTile>, grid_for(c, n, kCfTile), 256, 0, st, s.keys, inst, n, p.n_leaf,
                                                                             p.n_group, t.lv_tree, t.lv_grp);
     // groups
     SPH_TRY(scan_mode(c, t.lv_grp, nullptr, n, 1, c.d_sizes + SZ_GROUPS, st, t.grp_ref));
@@ -1210,10 +1233,10 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
     int nb = div_up(n, kChopBlock);
     int *blk_off = (int *)c.tmp1[2];
     int *ntotal = c.d_sizes + 2;
-    chop_count_kernel<<<nb, 256, 0, st>>>(t.lv_tree, n, t.blk_cnt, nb);
+    launch(chop_count_kernel, nb, 256, 0, st, t.lv_tree, n, t.blk_cnt, nb);
     SPH_TRY(scan_mode(c, t.blk_cnt, blk_off, kLevels * nb, 0, ntotal, st));
-    chop_write_kernel<<<nb, 256, 0, st>>>(t.lv_tree, n, blk_off, nb, ntotal, t, c.d_sizes, c.d_err);
-    node_finish_kernel<<<grid_for(c, node_cap_for(t, n), 256), 256, 0, st>>>(s.keys, inst, n, p.n_leaf, blk_off,
+    launch(chop_write_kernel, nb, 256, 0, st, t.lv_tree, n, blk_off, nb, ntotal, t, c.d_sizes, c.d_err);
+    launch(node_finish_kernel, grid_for(c, node_cap_for(t, n), 256), 256, 0, st, s.keys, inst, n, p.n_leaf, blk_off,
                                                                               nb, t, c.d_sizes);
     SPH_TRY(launch_bounds(c, s, 0, nullptr, st));
     return cudaGetLastError();
@@ -1222,6 +1245,7 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
 __global__ void pack_records_kernel(const float4 *__restrict__ pos, const float4 *__restrict__ vel,
                                     float4 *__restrict__ rec, int n)
 {
+    pdl_sync();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         rec[2 * (size_t)i] = pos[i];
         rec[2 * (size_t)i + 1] = vel[i];
@@ -1230,7 +1254,7 @@ __global__ void pack_records_kernel(const float4 *__restrict__ pos, const float4
 
 cudaError_t pack_records(Ctx &c, const sph_state &s, cudaStream_t st)
 {
-    pack_records_kernel<<<grid_for(c, s.n, 256), 256, 0, st>>>((const float4 *)s.pos,
+    launch(pack_records_kernel, grid_for(c, s.n, 256), 256, 0, st, (const float4 *)s.pos,
                                                                 (const float4 *)s.vel, c.rec, (int)s.n);
     return cudaGetLastError();
 }
@@ -1247,14 +1271,14 @@ cudaError_t update_hmax(Ctx &c, const sph_state &s, const sph_params &p, cudaStr
 // holds no keys (n = RS_TILE), so the block reads and writes no key; its
 // look-back polls tile 0's zeroed status word spin_cap times, raises
 // SPH_ERR_TIMEOUT in the error word and returns.
-__global__ void set_int_kernel(int *p, int v) { *p = v; }
+__global__ void set_int_kernel(int *p, int v) { pdl_sync(); *p = v; }
 
 cudaError_t sort_lookback_probe(Ctx &c, int spin_cap, cudaStream_t st)
 {
     // status words of tiles 0 and 1 (the buffer holds at least kRsSlots tiles)
     SPH_TRY(cudaMemsetAsync(c.rs_status, 0, sizeof(uint32_t) * 256 * 2, st));
-    set_int_kernel<<<1, 1, 0, st>>>(c.rs_tiles, 1);  // the block draws tile 1
-    rs_onesweep_kernel<<<1, RS_T, 0, st>>>(c.keys_alt, c.idx_a, c.keys_alt, c.idx_b, nullptr, RS_TILE,
+    launch(set_int_kernel, 1, 1, 0, st, c.rs_tiles, 1);  // the block draws tile 1
+    launch(rs_onesweep_kernel, 1, RS_T, 0, st, c.keys_alt, c.idx_a, c.keys_alt, c.idx_b, nullptr, RS_TILE,
                                           0, c.rs_gstart, c.rs_status, c.rs_tiles, c.d_err, nullptr,
                                           spin_cap);
     return cudaGetLastError();
