@@ -39,7 +39,7 @@ struct ForceSmem {
 
 struct ForceArgs {
     const float4 *pos, *vel, *prop;
-    const float4 *frec;  // [3 n] force records of the list kernel
+    const float4 *frec, *frec1, *frec2;  // [3 n] force records of the list kernel
     int tb;              // targets per batch of the list kernel (4, 8 or 16)
     float4 *acc;
     float *vsigmax;
@@ -159,10 +159,13 @@ struct ForceTarget {
 // (for M4, G = -3 and g_p(p) = max(1 - p, 0)^2 - max(1 - 2 p, 0)^2: the
 // derivative -3 q + 9/4 q^2 for q < 1, -3/4 (2 - q)^2 for 1 <= q < 2, 0
 // beyond).  With A = 1 / (rho Omega) and AK = G C A / h^4, A F = AK g_p.  A
-// neighbour is one 48-byte record (three 16-byte loads from one address):
+// neighbour is a record of three 16-byte words:
 // (x, y, z, m), (vx, vy, vz, (gamma - 1) u), ((R h)^2, AK, alpha c, rho).
 // The L1 data path is what bounds this kernel: the gathers deliver about
-// 48 bytes per wavefront, so the record holds only what the pair needs.
+// 48 bytes per wavefront, so the record holds only what the pair needs, and its
+// words lie in three arrays, where the neighbours of a warp's targets, close to
+// one another in curve order, share more lines than in 48-byte records (128^3
+// force stage 754 -> 734 us).
 // Per pair
 // (Eqs. 9-15, w = min(v_ij . rhat_ij, 0), hw = -w / 2):
 //   (P_i + q^i) / (rho_i^2 Omega_i) F_i = (P_i / rho_i + hw vsig_i) AK_i g_i
@@ -176,9 +179,8 @@ struct ForceSums {
     float ax, ay, az, sp, sv, sc, vsmax;
     int cnt;
 
-    __device__ __forceinline__ void init(const float4 *rec)
+    __device__ __forceinline__ void init(const float4 p, const float4 v, const float4 q)
     {
-        const float4 p = rec[0], v = rec[1], q = rec[2];
         xi = p.x; yi = p.y; zi = p.z;
         vxi = v.x; vyi = v.y; vzi = v.z; pri = v.w;
         R2i = q.x; AKi = q.y; aci = q.z; rhoi = q.w;
@@ -301,7 +303,7 @@ __global__ void __launch_bounds__(256, 3) force_list_kernel(ForceArgs a)
                     continue;
                 }
                 ForceSums<K, PER> T;
-                T.init(a.frec + 3 * (size_t)i);
+                T.init(a.frec[i], a.frec1[i], a.frec2[i]);
                 const int *__restrict__ lst = a.nl_idx + (size_t)i * a.nl_stride;
                 // Four consecutive entries per lane and iteration (one 16-byte
                 // load of the list, fetched an iteration ahead), no branch: an
@@ -310,8 +312,7 @@ __global__ void __launch_bounds__(256, 3) force_list_kernel(ForceArgs a)
                 // r = 0 would add nothing either (every term carries f'(0) = 0 or
                 // v_ij.r_ij / r = 0).
                 auto entry = [&](int j, bool valid) {
-                    const float4 *rj = a.frec + 3 * (size_t)j;
-                    T.pair(ld_keep(rj, 0, keep), ld_keep(rj, 1, keep), ld_keep(rj, 2, keep), valid,
+                    T.pair(ld_keep(a.frec, j, keep), ld_keep(a.frec1, j, keep), ld_keep(a.frec2, j, keep), valid,
                            a.beta, a.tree.per);
                 };
                 if (NPER == 4) {
@@ -490,7 +491,7 @@ __global__ void __launch_bounds__(kForceWarps * 32) force_walk_kernel(ForceArgs 
 __global__ void force_prep_kernel(const float4 *__restrict__ pos, const float4 *__restrict__ vel,
                                   const float *__restrict__ h, const float *__restrict__ rho,
                                   const float *__restrict__ omega, float4 *__restrict__ prop,
-                                  float4 *__restrict__ frec, int n, float gamma, float alpha, float kr,
+                                  float4 *__restrict__ frec, size_t stride, int n, float gamma, float alpha, float kr,
                                   float gc, float h_lim, int *err)
 {
     pdl_sync();
@@ -505,11 +506,7 @@ __global__ void force_prep_kernel(const float4 *__restrict__ pos, const float4 *
         const float cs = sqrtf(fmaxf(gamma * (gamma - 1.f) * v.w, 0.f));
         const float A = 1.f / (r * o);
         prop[i] = make_float4(hi, r, A, cs);
-        const float R = kr * hi;
-        const float hinv = 1.f / hi, hinv2 = hinv * hinv;
-        frec[3 * (size_t)i] = pos[i];
-        frec[3 * (size_t)i + 1] = make_float4(v.x, v.y, v.z, (gamma - 1.f) * v.w);
-        frec[3 * (size_t)i + 2] = make_float4(R * R, gc * A * hinv2 * hinv2, alpha * cs, r);
+        force_record(frec + i, stride, pos[i], v, hi, r, A, cs, gamma, alpha, kr, gc);
     }
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) raise_error(err, SPH_ERR_NONFINITE);
     if (__any_sync(0xffffffffu, neg) && (threadIdx.x & 31) == 0) raise_error(err, SPH_ERR_NEGATIVE_U);
@@ -602,11 +599,12 @@ cudaError_t configure_force_kernels(int kernel)
 cudaError_t force_prep(Ctx &c, const sph_state &s, const sph_params &p, cudaStream_t st,
                        bool hmax_now)
 {
+    if (prep_in_density(c)) return cudaSuccess;  // the density pass wrote the records
     const int n = (int)s.n;
     int grid = (n + 255) / 256;
     if (grid > c.num_sms * 16) grid = c.num_sms * 16;
     launch(force_prep_kernel, grid, 256, 0, st, (const float4 *)s.pos, (const float4 *)s.vel, s.h, s.rho,
-                                            s.omega, c.prop, c.frec, n, p.gamma, p.alpha_av,
+                                            s.omega, c.prop, c.frec, (size_t)c.max_n, n, p.gamma, p.alpha_av,
                                             kernel_support(p.kernel), kernel_gc(p.kernel),
                                             periodic_h_limit(p), c.d_err);
     cudaError_t e = cudaGetLastError();
@@ -661,6 +659,8 @@ cudaError_t force_pass(Ctx &c, const sph_state &s, const sph_params &p, cudaStre
     a.vel = (const float4 *)s.vel;
     a.prop = c.prop;
     a.frec = c.frec;
+    a.frec1 = c.frec + c.max_n;
+    a.frec2 = c.frec + 2 * c.max_n;
     a.acc = (float4 *)s.acc;
     a.vsigmax = s.vsigmax;
     a.drhodt = c.drhodt_in_force ? s.drhodt : nullptr;

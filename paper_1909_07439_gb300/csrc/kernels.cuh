@@ -135,6 +135,19 @@ struct SphKernel<2> {
     }
 };
 
+// The force record of a particle, three words: (x, y, z, m), (v, (gamma - 1) u),
+// ((R h)^2, G C / (h^4 rho Omega), alpha_AV c_s, rho); A = 1 / (rho Omega).  The
+// words lie in three arrays, `stride` apart.
+__device__ __forceinline__ void force_record(float4 *rec, size_t stride, float4 x, float4 v, float h, float rho, float A,
+                                             float cs, float gamma, float alpha, float kr, float gc)
+{
+    const float R = kr * h;
+    const float hinv = 1.f / h, hinv2 = hinv * hinv;
+    rec[0] = x;
+    rec[stride] = make_float4(v.x, v.y, v.z, (gamma - 1.f) * v.w);
+    rec[2 * stride] = make_float4(R * R, gc * A * hinv2 * hinv2, alpha * cs, rho);
+}
+
 // support radius, normalisation and G C of kernel k on the host
 inline float kernel_support(int k) { return k == 1 ? 3.f : 2.f; }
 inline float kernel_norm(int k)

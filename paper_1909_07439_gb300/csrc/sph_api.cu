@@ -180,7 +180,7 @@ sph_status do_density(Ctx &c, const sph_state &s, const sph_params &p, cudaStrea
 sph_status do_force(Ctx &c, const sph_state &s, const sph_params &p, cudaStream_t st,
                     bool records_fresh)
 {
-    {
+    if (!prep_in_density(c)) {
         StageScope sc(c, ST_PREP, st, kPrepLaunches + (records_fresh ? 0 : 1));
         CK(force_prep(c, s, p, st), "force_prep");
         if (!records_fresh) CK(pack_records(c, s, st), "pack");

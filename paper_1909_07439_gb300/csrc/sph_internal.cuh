@@ -135,8 +135,8 @@ struct Ctx {
     // per-particle scratch
     float4 *rec = nullptr;    // [2 n]: pos, vel of each particle side by side (32-byte records)
     float4 *prop = nullptr;   // h, rho, 1/(rho Omega), c_s
-    // [3 n]: the force record of each particle: (x, m), (v, (gamma - 1) u),
-    // ((R h)^2, G C / (h^4 rho Omega), alpha_AV c_s, rho)
+    // [3 n]: the force record of each particle, one array per word: (x, m), (v,
+    // (gamma - 1) u), ((R h)^2, G C / (h^4 rho Omega), alpha_AV c_s, rho)
     float4 *frec = nullptr;
     float4 *vhalf = nullptr;  // half-step v, u of the leapfrog
     // [n] block time steps: per-slot flag of the particles whose step ends in
@@ -356,6 +356,11 @@ struct DrhodtInForce {
     explicit DrhodtInForce(Ctx &cc) : c(cc) { c.drhodt_in_force = true; }
     ~DrhodtInForce() { c.drhodt_in_force = false; }
 };
+
+// Inside a step of all particles the density pass writes the force records (a
+// block step predicts the velocities of all particles anew for every substep,
+// and solves the density of the due ones only).
+inline bool prep_in_density(const Ctx &c) { return c.drhodt_in_force && !c.mask; }
 
 // lanes per target for a batch of nt targets (a power of two, nt * L <= 32)
 __host__ __device__ inline int lanes_per_target(int nt)
