@@ -86,19 +86,19 @@ __device__ __forceinline__ float seg_sum(float v, int L)
 
 // Sums of one pair at smoothing length 1/hinv (kernel K, whose f and f'
 // vanish beyond its support):
-//   s0 += m_j f(q), s1 += m_j (3 f + q f'), s2 += m_j vd f' / r
-// (h^3 rho = C s0, -h^4 d(rho)/dh = C s1, Eq. 3 numerator x h^4 / C = s2).
+//   s0 += m_j f(q) / F0, s1 += m_j (3 f + q f') / F1, s2 += m_j vd f' / r
+// (h^3 rho = C F0 s0, -h^4 d(rho)/dh = C F1 s1, Eq. 3 numerator x h^4 / C = s2).
 template <int K, bool VD = true>
 __device__ __forceinline__ void pair_sums(float r2, float mj, float vd, float hinv, float &s0,
                                           float &s1, float &s2)
 {
     // r = 0 (the particle itself, or a padding entry) gives q = 0 and vd = 0
-    const float rinv = rsqrtf(fmaxf(r2, 1e-30f));
+    const float rinv = rsqrt_normal(fmaxf(r2, 1e-30f));
     const float q = r2 * rinv * hinv;
-    float f, df;
-    SphKernel<K>::f_df(q, f, df);
+    float f, g, df;
+    SphKernel<K>::sums(q, f, g, df);
     s0 += mj * f;
-    s1 += mj * (3.f * f + q * df);
+    s1 += mj * g;
     if (VD) s2 += mj * vd * df * rinv;
 }
 
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
                     // lists come from DRAM), no branch on the distance: f and f'
                     // vanish for q >= R, so entries beyond R h add nothing.  A
                     // missing entry repeats the first with zero mass.
-                    auto entry = [&](float4 pj, float4 vj, float mj) {
+                    auto entry = [&](float4 pj, float4 vj, float mj, bool real) {
                         float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
                         if (PER) {  // nearest images on the periodic axes
                             dx = wrap_sep(dx, a.tree.per.x);
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
                         const float r2 = dx * dx + dy * dy + dz * dz;
                         const float vd =
                             VD ? (vi.x - vj.x) * dx + (vi.y - vj.y) * dy + (vi.z - vj.z) * dz : 0.f;
-                        cnt += (mj > 0.f && r2 < R2) ? 1 : 0;
+                        cnt += (real && r2 < R2) ? 1 : 0;
                         pair_sums<K, VD>(r2, mj, vd, hinv, s0, s1, s2);
                     };
                     // neighbour j's position (and velocity with VD)
@@ -270,10 +270,10 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
                             load(b1 ? jj.y : jj.x, p1, v1);
                             load(b2 ? jj.z : jj.x, p2, v2);
                             load(b3 ? jj.w : jj.x, p3, v3);
-                            entry(p0, v0, p0.w);
-                            entry(p1, v1, b1 ? p1.w : 0.f);
-                            entry(p2, v2, b2 ? p2.w : 0.f);
-                            entry(p3, v3, b3 ? p3.w : 0.f);
+                            entry(p0, v0, p0.w, true);
+                            entry(p1, v1, b1 ? p1.w : 0.f, b1);
+                            entry(p2, v2, b2 ? p2.w : 0.f, b2);
+                            entry(p3, v3, b3 ? p3.w : 0.f, b3);
                         }
                     } else {
                         int e = 2 * sub;
@@ -285,12 +285,12 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
                             float4 p0, v0, p1, v1;
                             load(jj.x, p0, v0);
                             load(b1 ? jj.y : jj.x, p1, v1);
-                            entry(p0, v0, p0.w);
-                            entry(p1, v1, b1 ? p1.w : 0.f);
+                            entry(p0, v0, p0.w, true);
+                            entry(p1, v1, b1 ? p1.w : 0.f, b1);
                         }
                     }
-                    s0 = seg_sum(s0, L);
-                    s1 = seg_sum(s1, L);
+                    s0 = SphKernel<K>::F0 * seg_sum(s0, L);
+                    s1 = SphKernel<K>::F1 * seg_sum(s1, L);
                     s2 = seg_sum(s2, L);
                     const float cf = seg_sum((float)cnt, L);
                     if (sub == 0 && on) {
@@ -499,8 +499,8 @@ __global__ void __launch_bounds__(kDensWarps * 32, 4) density_walk_kernel(DensAr
                 } else {
                     list_sums();
                 }
-                s0 = seg_sum(s0, L);
-                s1 = seg_sum(s1, L);
+                s0 = SphKernel<K>::F0 * seg_sum(s0, L);
+                s1 = SphKernel<K>::F1 * seg_sum(s1, L);
                 s2 = seg_sum(s2, L);
                 const float cf = seg_sum((float)cnt, L);
                 if (sub == 0 && on) {

@@ -207,9 +207,9 @@ struct ForceSums {
         // r < R max(h_i, h_j) as r^2 < max((R h_i)^2, (R h_j)^2): squaring is monotone
         const bool in = valid && r2 > 0.f && r2 < fmaxf(R2i, q.x);
         const float mj = in ? p.w : 0.f;
-        const float rinv = rsqrtf(fmaxf(r2, 1e-30f));
+        const float rinv = rsqrt_normal(fmaxf(r2, 1e-30f));
         const float r = r2 * rinv;
-        const float pi = r * rsqrtf(R2i), pj = r * rsqrtf(q.x);   // q / R of each side
+        const float pi = r * rsqrt_normal(R2i), pj = r * rsqrt_normal(q.x);   // q / R of each side
         const float gi = SphKernel<K>::g_p(pi), gj = SphKernel<K>::g_p(pj);
         const float Ti = AKi * gi, Tj = q.y * gj;
         const float dvx = vxi - v.x, dvy = vyi - v.y, dvz = vzi - v.z, dpr = pri - prj;
@@ -227,7 +227,7 @@ struct ForceSums {
         sp = fmaf(mg, vr, sp);
         sv = fmaf(mg, vsi * (hw * hw), sv);
         const float dP = fabsf(Pi - prj * q.w);
-        const float vu = dP * rsqrtf(fmaxf(dP * (rhoi + q.w), 1e-30f));
+        const float vu = dP * rsqrt_normal(fmaxf(dP * (rhoi + q.w), 1e-30f));
         sc = fmaf(mj * (vu * dpr), Ti + Tj, sc);
         vsmax = fmaxf(vsmax, in ? vsi : 0.f);
         cnt += in ? 1 : 0;

@@ -21,6 +21,8 @@
 //              a   = -M d / r^3 + Q d / r^5 - 5 (d.Q.d) d / (2 r^7)
 //   particle:  phi = -m/r,  a = -m d / r^3
 // with d = x_i - X (or x_i - x_j) and r^2 = |d|^2 + eps^2.  FP32 throughout.
+#include <algorithm>
+
 #include "kernels.cuh"
 #include "walk.cuh"
 
@@ -197,7 +199,7 @@ __global__ void __launch_bounds__(kGWarps * 32) gravity_kernel(GravArgs a)
                 const float2 qzz = make_float2(Q1.x, Q1.y), qxy = make_float2(Q1.z, Q1.w);
                 const float2 qxz = make_float2(Q2.x, Q2.y), qyz = make_float2(Q2.z, Q2.w);
                 const float2 r2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, e2)));
-                const float2 rinv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+                const float2 rinv = make_float2(rsqrt_normal(r2.x), rsqrt_normal(r2.y));
                 const float2 rinv2 = mul2(rinv, rinv), rinv3 = mul2(rinv, rinv2), rinv5 = mul2(rinv3, rinv2);
                 const float2 qx = fma2(qxx, dx, fma2(qxy, dy, mul2(qxz, dz)));
                 const float2 qy = fma2(qxy, dx, fma2(qyy, dy, mul2(qyz, dz)));
@@ -231,7 +233,7 @@ __global__ void __launch_bounds__(kGWarps * 32) gravity_kernel(GravArgs a)
                 const float2 dy = add2(make_float2(A.z, A.w), mul2(ty, f2(-1.f)));
                 const float2 dz = add2(make_float2(B.x, B.y), mul2(tz, f2(-1.f)));
                 const float2 r2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, e2)));
-                const float2 rinv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+                const float2 rinv = make_float2(rsqrt_normal(r2.x), rsqrt_normal(r2.y));
                 const float2 mr = mul2(m, rinv);
                 const float2 mr3 = mul2(mr, mul2(rinv, rinv));
                 ax2 = fma2(mr3, dx, ax2);
@@ -425,7 +427,7 @@ cudaError_t gravity_pass(Ctx &c, const sph_state &s, const sph_params &p, float4
     a.acc = acc;
     a.out = out;
     a.G = p.grav_G;
-    a.eps2 = p.grav_eps * p.grav_eps;
+    a.eps2 = std::max(p.grav_eps * p.grav_eps, 1.2e-38f);  // r^2 stays normal
     a.err = c.d_err;
     a.counters = c.d_counters;
     (void)n;
