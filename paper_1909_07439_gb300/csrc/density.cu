@@ -29,7 +29,7 @@ namespace sph {
 constexpr int kTB = kWalkTB;     // targets per batch of the walking kernel
 constexpr int kDensWarps = 4;    // warps per block
 constexpr float kPad = kListPad; // padded list radius, relative to h
-constexpr int kRound = 2;        // groups per warp per work grab of the list kernel
+constexpr int kRound = 2;        // groups per warp per work grab of the list kernel (1 in a small tree)
 
 template <int CAP>
 struct DensSmem {
@@ -185,20 +185,25 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
     const float hf3 = a.hfact * a.hfact * a.hfact;
     const bool fixed = a.fixed_iters > 0;
     const int limit = fixed ? a.fixed_iters : a.max_iter;
-    unsigned long long n_pairs = 0, n_newton = 0;
+    unsigned n_pairs = 0, n_newton = 0;  // a lane's share of a launch stays far below 2^32
     // The block takes kRound consecutive groups per warp at a time, warp w the
     // groups base + w + nw k: the warps of a block work on neighbouring groups
     // together and share their candidates in L1.
     __shared__ int s_base;
     const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 
+    // one at a time while two would leave warps without a group, or the last
+    // round of grabs nearly empty (2003 particles 28.8 -> 21.5 us, 8192 155 -> 138,
+    // the 165888 of a tube 312 -> 304; 128^3 keeps two)
+    __shared__ int s_round;
+    if (threadIdx.x == 0) s_round = ng < kSmallRounds * kRound * nw * (int)gridDim.x ? 1 : kRound;
     while (true) {
-        if (threadIdx.x == 0) s_base = atomicAdd(a.work, nw * kRound);
+        if (threadIdx.x == 0) s_base = atomicAdd(a.work, nw * s_round);
         __syncthreads();
         const int base = s_base;
         __syncthreads();
         if (base >= ng) break;
-        for (int kr = 0; kr < kRound; ++kr) {
+        for (int kr = 0; kr < s_round; ++kr) {
             const int gq = base + warp + nw * kr;
             if (gq >= ng) break;
             const int g = ng - 1 - gq;  // last group first: its lists were written last (in L2)
@@ -294,7 +299,7 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
                     s2 = seg_sum(s2, L);
                     const float cf = seg_sum((float)cnt, L);
                     if (sub == 0 && on) {
-                        n_pairs += (unsigned long long)cf;
+                        n_pairs += (unsigned)cf;
                         ++n_newton;
                     }
                     if (final_pass) break;
@@ -321,13 +326,14 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
             }
         }
     }
+    unsigned long long pairs = n_pairs, newton = n_newton;
     for (int o = 16; o > 0; o >>= 1) {
-        n_pairs += __shfl_xor_sync(0xffffffffu, n_pairs, o);
-        n_newton += __shfl_xor_sync(0xffffffffu, n_newton, o);
+        pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+        newton += __shfl_xor_sync(0xffffffffu, newton, o);
     }
     if (lane == 0) {
-        atomicAdd(&a.counters[C_DENS_PAIRS], n_pairs);
-        atomicAdd(&a.counters[C_NEWTON], n_newton);
+        atomicAdd(&a.counters[C_DENS_PAIRS], pairs);
+        atomicAdd(&a.counters[C_NEWTON], newton);
     }
 }
 

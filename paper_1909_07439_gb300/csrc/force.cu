@@ -23,7 +23,7 @@ namespace sph {
 
 constexpr int kFTB = kWalkTB;    // targets per batch of the walking kernel
 constexpr int kForceWarps = 4;   // warps per block
-constexpr int kRound = 2;        // groups per warp per work grab of the list kernel
+constexpr int kRound = 2;        // groups per warp per work grab of the list kernel (1 in a small tree)
 
 template <int CAP>
 struct ForceSmem {
@@ -269,20 +269,25 @@ __global__ void __launch_bounds__(256, 3) force_list_kernel(ForceArgs a)
     const uint64_t keep = l2_keep_policy();
     const int ng = a.sizes[SZ_GROUPS];
     const bool lists_fresh = a.rec_ctl[1] == 0;
-    unsigned long long n_pairs = 0, n_cand = 0, n_fb = 0;
+    unsigned n_pairs = 0, n_cand = 0, n_fb = 0;  // a lane's share of a launch stays far below 2^32
     // The block takes kRound consecutive groups per warp at a time, warp w the
     // groups base + w + nw k: the warps of a block work on neighbouring groups
     // together and share their candidates in L1.
     __shared__ int s_base;
     const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 
+    // one at a time while two would leave warps without a group, or the last
+    // round of grabs nearly empty (2003 particles 35.9 -> 31.0 us, 8192 76 -> 71;
+    // 128^3 keeps two)
+    __shared__ int s_round;
+    if (threadIdx.x == 0) s_round = ng < kSmallRounds * kRound * nw * (int)gridDim.x ? 1 : kRound;
     while (true) {
-        if (threadIdx.x == 0) s_base = atomicAdd(a.work, nw * kRound);
+        if (threadIdx.x == 0) s_base = atomicAdd(a.work, nw * s_round);
         __syncthreads();
         const int base = s_base;
         __syncthreads();
         if (base >= ng) break;
-        for (int kr = 0; kr < kRound; ++kr) {
+        for (int kr = 0; kr < s_round; ++kr) {
             const int g = base + warp + nw * kr;
             if (g >= ng) break;
             const int2 gr = a.grp_ref[g];
@@ -340,18 +345,19 @@ __global__ void __launch_bounds__(256, 3) force_list_kernel(ForceArgs a)
                 }
                 T.finish(L, on && sub == 0, i, a.gm1, a.alpha_u, a.acc, a.vsigmax, a.drhodt);
                 n_pairs += on ? T.cnt : 0;
-                n_cand += on && sub == 0 ? (unsigned long long)len : 0ull;
+                n_cand += on && sub == 0 ? len : 0;
             }
         }
     }
+    unsigned long long pairs = n_pairs, cand = n_cand;
     for (int o = 16; o > 0; o >>= 1) {
-        n_pairs += __shfl_xor_sync(0xffffffffu, n_pairs, o);
-        n_cand += __shfl_xor_sync(0xffffffffu, n_cand, o);
+        pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+        cand += __shfl_xor_sync(0xffffffffu, cand, o);
     }
     if (lane == 0) {
-        atomicAdd(&a.counters[C_FORCE_PAIRS], n_pairs);
-        atomicAdd(&a.counters[C_FORCE_CAND], n_cand);
-        if (n_fb) atomicAdd(&a.counters[C_FORCE_FB], n_fb);  // warp-uniform count
+        atomicAdd(&a.counters[C_FORCE_PAIRS], pairs);
+        atomicAdd(&a.counters[C_FORCE_CAND], cand);
+        if (n_fb) atomicAdd(&a.counters[C_FORCE_FB], (unsigned long long)n_fb);  // warp-uniform count
     }
 }
 

@@ -223,7 +223,8 @@ inline float3 box_lo_of(const sph_params &p) { return make_float3(p.box_lo[0], p
 // up while the last blocks of that kernel still run, wait there until it has
 // finished and its writes are visible, and then let the next kernel's blocks be
 // set up.  A step is some 40 short kernels that each depend on the one before:
-// PDLMEAS
+// a step of 2003 particles 249 -> 232 us, of 8192 450 -> 420, an 8-step rollout
+// of 64^3 and its adjoint 45.1 -> 40.2 ms.
 __device__ __forceinline__ void pdl_sync()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -367,6 +368,9 @@ __host__ __device__ inline int lanes_per_target(int nt)
 {
     return nt > 8 ? 2 : nt > 4 ? 4 : nt > 2 ? 8 : nt > 1 ? 16 : 32;
 }
+
+// rounds of grabs below which the pair kernels take one group per warp at a time
+constexpr int kSmallRounds = 8;
 
 // number of blocks used by the chop's per-block counting (1024 particles each)
 constexpr int kChopBlock = 1024;
