@@ -21,16 +21,18 @@ class DeviceState:
     FIELDS4 = ("pos", "vel", "acc")
     FIELDS1 = ("h", "rho", "omega", "drhodt", "vsigmax")
 
-    def __init__(self, n: int, device="cuda"):
+    def __init__(self, n: int, device="cuda", zero=True):
+        """zero=False: the arrays' contents are undefined (perm excepted)."""
         import torch
         self.n = int(n)
         self.device = torch.device(device)
-        z4 = lambda: torch.zeros((max(self.n, 1), 4), dtype=torch.float32, device=self.device)
-        z1 = lambda: torch.zeros(max(self.n, 1), dtype=torch.float32, device=self.device)
+        make = torch.zeros if zero else torch.empty
+        z4 = lambda: make((max(self.n, 1), 4), dtype=torch.float32, device=self.device)
+        z1 = lambda: make(max(self.n, 1), dtype=torch.float32, device=self.device)
         self.pos, self.vel, self.acc = z4(), z4(), z4()
         self.h, self.rho, self.omega, self.drhodt, self.vsigmax = z1(), z1(), z1(), z1(), z1()
         self.perm = torch.arange(max(self.n, 1), dtype=torch.int32, device=self.device)
-        self.keys = torch.zeros(max(self.n, 1), dtype=torch.int64, device=self.device)
+        self.keys = make(max(self.n, 1), dtype=torch.int64, device=self.device)
 
     @classmethod
     def from_arrays(cls, pos, vel, h, device="cuda"):
