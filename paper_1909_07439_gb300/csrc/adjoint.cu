@@ -59,9 +59,12 @@ struct PairWalkSmem {
     int ej[kPW_TB][CAP];
 };
 
+// Five blocks per SM: the gathers' latency is what binds, and a rollout of 8 steps of
+// 64^3 with its adjoint took 39.0 -> 38.3 ms although the force operator spills
+// some 60 bytes at that limit.
 // Op: struct with  Acc;  init(i, Acc&);  pair(j, x_j and m_j, Acc&);  reduce(Acc&, L);  store(i, Acc&)
 template <int CAP, class Op>
-__global__ void __launch_bounds__(128) pairwalk_kernel(PairWalkArgs a, Op op)
+__global__ void __launch_bounds__(128, 5) pairwalk_kernel(PairWalkArgs a, Op op)
 {
     pdl_sync();
     extern __shared__ __align__(16) unsigned char pw_raw[];
@@ -184,10 +187,11 @@ __global__ void __launch_bounds__(128) pairwalk_kernel(PairWalkArgs a, Op op)
 // difference of the rounded products is exact (Sterbenz), so the difference
 // keeps about twice FP32's precision.  The conduction speed's derivative
 // carries 1 / sqrt(|P_i - P_j|), so the difference must not be swamped by
-// the rounding of the two pressures.
+// the rounding of the two pressures.  (The products by intrinsics, which the
+// compiler never contracts: a - b as one FMA would count ea twice, 1e-3 of dL/du.)
 __device__ __forceinline__ float pressure_diff(float gm1, float ri, float ui, float rj, float uj)
 {
-    const float a = ri * ui, b = rj * uj;
+    const float a = __fmul_rn(ri, ui), b = __fmul_rn(rj, uj);
     const float ea = fmaf(ri, ui, -a), eb = fmaf(rj, uj, -b);
     return gm1 * ((a - b) + (ea - eb));
 }
