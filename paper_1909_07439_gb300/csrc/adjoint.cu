@@ -528,7 +528,7 @@ static cudaError_t launch_pairwalk(Ctx &c, const sph_state &s, bool dens_set, fl
     a.rec_ctl = c.tree.rec_ctl;
     a.rec_bad = c.tree.rec_bad;
     a.err = c.d_err;
-    cudaError_t e = cudaMemsetAsync(a.work, 0, sizeof(int), st);
+    cudaError_t e = clear_words(Clear{{a.work}, {1}}, st);
     if (e != cudaSuccess) return e;
     launch(pairwalk_kernel<CAP, Op>, c.num_sms * blocks, 128, smem, st, a, op);
     return cudaGetLastError();

@@ -796,16 +796,20 @@ static cudaError_t density_solve_k(Ctx &c, DensArgs &a, const sph_params &p, cud
     const int wl = ps.warps == 8 ? 3 : ps.warps == 4 ? 2 : ps.warps == 2 ? 1 : 0;
     const dim3 grid(c.num_sms * bl[wl]), block(32 * ps.warps);
     const bool per = a.tree.per.any();
+    // Not a programmatic dependent: its blocks would settle on an SM beside the list
+    // build's last ones, whose 220 KB of shared memory leave little L1, and an SM
+    // divides the two anew only when it is empty.  (Chained, a step of 128^3 2.90 ms
+    // instead of 2.67, of 64^3 596 us instead of 589; of 2003 particles 121 and 118.)
     if (a.vd) {
-        if (ps.unroll == 4 && per) launch(density_list_kernel<4, K, true, true>, grid, block, 0, st, a);
-        else if (ps.unroll == 4) launch(density_list_kernel<4, K, false, true>, grid, block, 0, st, a);
-        else if (per) launch(density_list_kernel<2, K, true, true>, grid, block, 0, st, a);
-        else launch(density_list_kernel<2, K, false, true>, grid, block, 0, st, a);
+        if (ps.unroll == 4 && per) launch<false>(density_list_kernel<4, K, true, true>, grid, block, 0, st, a);
+        else if (ps.unroll == 4) launch<false>(density_list_kernel<4, K, false, true>, grid, block, 0, st, a);
+        else if (per) launch<false>(density_list_kernel<2, K, true, true>, grid, block, 0, st, a);
+        else launch<false>(density_list_kernel<2, K, false, true>, grid, block, 0, st, a);
     } else {
-        if (ps.unroll == 4 && per) launch(density_list_kernel<4, K, true, false>, grid, block, 0, st, a);
-        else if (ps.unroll == 4) launch(density_list_kernel<4, K, false, false>, grid, block, 0, st, a);
-        else if (per) launch(density_list_kernel<2, K, true, false>, grid, block, 0, st, a);
-        else launch(density_list_kernel<2, K, false, false>, grid, block, 0, st, a);
+        if (ps.unroll == 4 && per) launch<false>(density_list_kernel<4, K, true, false>, grid, block, 0, st, a);
+        else if (ps.unroll == 4) launch<false>(density_list_kernel<4, K, false, false>, grid, block, 0, st, a);
+        else if (per) launch<false>(density_list_kernel<2, K, true, false>, grid, block, 0, st, a);
+        else launch<false>(density_list_kernel<2, K, false, false>, grid, block, 0, st, a);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -826,11 +830,6 @@ cudaError_t density_lists(Ctx &c, const sph_state &s, const sph_params &p, cudaS
     cudaError_t e = cudaSuccess;
     // node and group h_max of the starting h: the list walk's opening test needs them
     if (refresh_hmax) e = update_hmax(c, s, p, st);
-    if (e != cudaSuccess) return e;
-    // fresh lists: valid unless an h outgrows its pad
-    e = cudaMemsetAsync(c.tree.rec_ctl, 0, 2 * sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(c.tree.rec_bad, 0, sizeof(int) * (batch ? batch->n_inst : 1), st);
     if (e != cudaSuccess) return e;
     c.nl_kernel = p.kernel;
     c.nl_stride = list_cap(p.kernel);
@@ -880,9 +879,7 @@ cudaError_t density_solve(Ctx &c, const sph_state &s, const sph_params &p, cudaS
     a.fixed_iters = p.density_iters;
     a.err = c.d_err;
     a.counters = c.d_counters;
-    static_assert(SZ_FALLBACK == SZ_WORK + 1 && SZ_WORK2 == SZ_WORK + 2, "work counters adjacent");
-    cudaError_t e = cudaMemsetAsync(a.work, 0, 3 * sizeof(int), st);
-    if (e != cudaSuccess) return e;
+    // (the list build zeroed the work counters)
     if (p.kernel == 1) return density_solve_k<1>(c, a, p, st);
     if (p.kernel == 2) return density_solve_k<2>(c, a, p, st);
     return density_solve_k<0>(c, a, p, st);

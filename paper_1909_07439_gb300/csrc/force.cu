@@ -686,9 +686,8 @@ cudaError_t force_pass(Ctx &c, const sph_state &s, const sph_params &p, cudaStre
     e = check_list_kernel(c, p, st);
     if (e != cudaSuccess) return e;
     // lists of instances where an h outgrew the pad are rebuilt at the final h
+    // (the pass also zeroes the work counters)
     e = relist_pass(c, s, p, kListPad, st, batch);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(a.work, 0, 3 * sizeof(int), st);  // work, fallback count, work2
     if (e != cudaSuccess) return e;
     if (p.kernel == 1) return force_launch_k<1>(c, a, p, s, st);
     if (p.kernel == 2) return force_launch_k<2>(c, a, p, s, st);

@@ -75,6 +75,7 @@ struct NlistArgs {
     const float4 *grp_lo, *grp_hi;
     const int *sizes;
     int *work;
+    int *pair_work;  // [3] work counters of the density and force kernels: zeroed for the one that follows
     WalkTree tree;
     const int *inst;
     float rscale;  // list radius = rscale * max(h_i, h_j)
@@ -304,6 +305,7 @@ __global__ void __launch_bounds__(kNlWarps * 32, 7) nlist_kernel(NlistArgs a)
     const int lane = threadIdx.x & 31;
     const unsigned lt = lane_lt();
     const int ng = a.sizes[SZ_GROUPS];
+    if (blockIdx.x == 0 && threadIdx.x < 3) a.pair_work[threadIdx.x] = 0;
     if (a.gate && *a.gate == 0) return;  // relist mode, nothing outgrew its pad
     // per-warp tallies (32 bits: a warp's share of a launch stays far below 2^32)
     unsigned n_cand = 0, n_entries = 0, n_over = 0;
@@ -514,7 +516,9 @@ static NlistArgs nlist_args(Ctx &c, const sph_state &s, const sph_params &p, flo
     a.grp_lo = c.tree.grp_lo;
     a.grp_hi = c.tree.grp_hi;
     a.sizes = c.d_sizes;
-    a.work = c.d_sizes + SZ_WORK;
+    a.work = c.d_sizes + SZ_NL;
+    static_assert(SZ_FALLBACK == SZ_WORK + 1 && SZ_WORK2 == SZ_WORK + 2, "work counters adjacent");
+    a.pair_work = c.d_sizes + SZ_WORK;
     a.tree = WalkTree{c.tree.node_lo, c.tree.node_hi, c.tree.node_ref, period_of(p)};
     a.inst = batch ? c.inst : nullptr;
     // the radius and capacity of the lists' kernel (a relist keeps them)
@@ -534,9 +538,11 @@ cudaError_t nlist_pass(Ctx &c, const sph_state &s, const sph_params &p, float pa
     int blocks = 1;
     cudaError_t e = configure_nlist(blocks);
     if (e != cudaSuccess) return e;
-    NlistArgs a = nlist_args(c, s, p, pad, batch);
-    e = cudaMemsetAsync(a.work, 0, sizeof(int), st);
+    // fresh lists: valid unless an h outgrows its pad
+    static_assert(SZ_NL2 == SZ_NL + 1, "list work counters adjacent");
+    e = clear_words(Clear{{c.tree.rec_ctl, c.tree.rec_bad, c.d_sizes + SZ_NL}, {2, batch ? batch->n_inst : 1, 2}}, st);
     if (e != cudaSuccess) return e;
+    const NlistArgs a = nlist_args(c, s, p, pad, batch);
     return launch_nlist(c, a, blocks, st);
 }
 
@@ -557,16 +563,13 @@ cudaError_t relist_pass(Ctx &c, const sph_state &s, const sph_params &p, float p
     e = update_hmax(c, s, p, st, any);
     if (e != cudaSuccess) return e;
     NlistArgs a = nlist_args(c, s, p, pad, batch);
+    a.work = c.d_sizes + SZ_NL2;
     a.gate = any;
     a.only_bad = c.tree.rec_bad;
-    e = cudaMemsetAsync(a.work, 0, sizeof(int), st);
-    if (e != cudaSuccess) return e;
     e = launch_nlist(c, a, blocks, st);
     if (e != cudaSuccess) return e;
     // the rebuilt lists cover the pair sets at the final h
-    e = cudaMemsetAsync(c.tree.rec_bad, 0, sizeof(int) * (batch ? batch->n_inst : 1), st);
-    if (e != cudaSuccess) return e;
-    return cudaMemsetAsync(any, 0, sizeof(int), st);
+    return clear_words(Clear{{c.tree.rec_bad, any, a.work}, {batch ? batch->n_inst : 1, 1, 1}}, st);
 }
 
 }  // namespace sph

@@ -167,7 +167,7 @@ sph_status do_density(Ctx &c, const sph_state &s, const sph_params &p, cudaStrea
         CK(pack_records(c, s, st), "pack");
     }
     {
-        StageScope sc(c, ST_LISTS, st, 1);
+        StageScope sc(c, ST_LISTS, st, 2);
         CK(density_lists(c, s, p, st, nullptr, false), "neighbour lists");
     }
     StageScope sc(c, ST_DENSITY, st, 2);
@@ -187,7 +187,7 @@ sph_status do_force(Ctx &c, const sph_state &s, const sph_params &p, cudaStream_
     }
     {
         // relist (h_max refresh, list kernel), list kernel, h_max refresh, walking fallback
-        StageScope sc(c, ST_FORCE, st, 5);
+        StageScope sc(c, ST_FORCE, st, 6);
         CK(force_pass(c, s, p, st), "force");
     }
     if (p.grav_G > 0.f) {
@@ -400,9 +400,8 @@ sph_status sph_create(sph_ctx **out, int64_t max_n, int device)
     A(dalloc(c.idx_a, n));
     A(dalloc(c.idx_b, n));
     A(dalloc(c.rs_ghist, 10 * 256));
-    A(dalloc(c.rs_gstart, 10 * 256));
     A(dalloc(c.rs_status, (size_t)kRsSlots * 256 * c.ntiles_cap));
-    A(dalloc(c.rs_tiles, kRsSlots + 1));
+    A(dalloc(c.rs_tiles, kRsSlots + kRsFlags));
     for (int k = 0; k < 4; ++k) A(dalloc(c.tmp4[k], n));
     for (int k = 0; k < 5; ++k) A(dalloc(c.tmp1[k], n));
     A(dalloc(c.tmp_perm, n));
@@ -467,7 +466,7 @@ void sph_destroy(sph_ctx *h)
     cudaSetDevice(c.device);
     cudaDeviceSynchronize();
     release_rollout(c);
-    void *ptrs[] = {c.keys_alt, c.idx_a, c.idx_b, c.rs_ghist, c.rs_gstart, c.rs_status, c.rs_tiles, c.tmp4[0], c.tmp4[1], c.tmp4[2],
+    void *ptrs[] = {c.keys_alt, c.idx_a, c.idx_b, c.rs_ghist, c.rs_status, c.rs_tiles, c.tmp4[0], c.tmp4[1], c.tmp4[2],
                     c.tmp4[3], c.tmp1[0], c.tmp1[1], c.tmp1[2], c.tmp1[3], c.tmp1[4], c.tmp_perm,
                     c.tree.node_first, c.tree.node_count, c.tree.node_level, c.tree.node_child,
                     c.tree.node_nchild, c.tree.node_parent, c.tree.node_arrive, c.tree.node_lo,

@@ -17,6 +17,9 @@ constexpr int kMaxLevel = 21;        // 21 bits per axis, 63-bit keys
 constexpr int kLevels = 22;          // levels 0..21
 constexpr int kWarp = 32;
 constexpr int kMaxInstances = 65536;  // instances in one batch
+// flags of a sort, after its tile counters: RF_FULL, the fix-up found a long run
+// (all 64 bits are sorted); RF_UNSORTED, the keys were not in order already
+enum { RF_FULL = 0, RF_UNSORTED = 1, kRsFlags = 2 };
 constexpr int kRsSlots = 14;         // radix passes of one sort at most (4 + 8 + 2)
 // Neighbour-list entries per particle (also the lists' stride): at least
 // twice the mean list length of the kernel at its usual hfact (list radius
@@ -60,8 +63,9 @@ enum Counter {
 // tree-size scalars on the device (Ctx::d_sizes)
 // SZ_WORK / SZ_WORK2: work counters of the persistent kernels; SZ_FALLBACK:
 // entries in Ctx::fallback; SZ_BAD_OFFSETS: the batch offsets failed their check
+// SZ_NL / SZ_NL2: work counters of the list build and of the relist
 enum Size { SZ_NODES = 0, SZ_GROUPS = 1, SZ_WORK = 3, SZ_FALLBACK = 4, SZ_WORK2 = 5, SZ_BAD_OFFSETS = 6,
-            SZ_N = 8 };
+            SZ_NL = 8, SZ_NL2 = 9, SZ_N = 12 };
 
 struct Tree {
     int cap_nodes = 0;
@@ -104,9 +108,8 @@ struct Ctx {
     uint64_t *keys_alt = nullptr;
     uint32_t *idx_a = nullptr, *idx_b = nullptr;
     uint32_t *rs_ghist = nullptr;   // [10][256] digit counts of every pass
-    uint32_t *rs_gstart = nullptr;  // [10][256] their exclusive scans
     uint32_t *rs_status = nullptr;  // [kRsSlots][ntiles][256] look-back words, one slot per pass
-    int *rs_tiles = nullptr;        // [kRsSlots] tile counters, then the full-sort flag
+    int *rs_tiles = nullptr;        // [kRsSlots] tile counters, then the flags of rs_flag
     int ntiles_cap = 0;
 
     // gather scratch
@@ -231,7 +234,8 @@ __device__ __forceinline__ void pdl_sync()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-template <class... P, class... A>
+// CHAIN = false: an ordinary launch, after everything before it
+template <bool CHAIN = true, class... P, class... A>
 inline cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
 {
     cudaLaunchAttribute at{};
@@ -243,7 +247,7 @@ inline cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t sm
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = CHAIN ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
@@ -266,6 +270,14 @@ cudaError_t scan_exclusive_int(Ctx &c, const int *in, int *out, int n, int *tota
 // test hook: a sort pass whose look-back predecessor never publishes
 cudaError_t sort_lookback_probe(Ctx &c, int spin_cap, cudaStream_t st);
 // nlist.cu
+// Zeros up to three ranges of words with one kernel: a memset in its place would
+// end the chain of programmatic dependents.
+struct Clear {
+    int *p[3];
+    int n[3];
+};
+cudaError_t clear_words(const Clear &z, cudaStream_t st);
+
 cudaError_t nlist_pass(Ctx &c, const sph_state &s, const sph_params &p, float pad,
                        cudaStream_t st, const Batch *batch = nullptr);
 // After the density pass: rebuild, at the final h, the lists of the

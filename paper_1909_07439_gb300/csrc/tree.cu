@@ -51,11 +51,29 @@ __device__ __forceinline__ uint64_t spread21(uint32_t v)
 }
 
 // ------------------------------------------------------------ bbox + checks
-__global__ void bbox_init_kernel(int *bb)
+// What a build starts from, in one kernel instead of four memsets (which would
+// end the chain of programmatic dependents): the boxes (six ordered ints each),
+// zeroed digit counts, tile counters, flags and look-back words of the radix
+// sort, and lists marked stale (they refer to the previous tree).
+struct BuildInit {
+    int *bb;
+    int nbox;
+    uint4 *hist, *status;
+    int nhist, nstatus;  // in 16-byte words
+    int *tiles;
+    int ntiles;
+    int *stale;
+};
+__global__ void build_init_kernel(BuildInit a)
 {
     pdl_sync();
-    if (threadIdx.x < 3) bb[threadIdx.x] = 0x7fffffff;           // min of ordered ints
-    else if (threadIdx.x < 6) bb[threadIdx.x] = (int)0x80000000; // max
+    const int t0 = blockIdx.x * blockDim.x + threadIdx.x, dt = gridDim.x * blockDim.x;
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+    for (int k = t0; k < a.nstatus; k += dt) a.status[k] = z;
+    for (int k = t0; k < a.nhist; k += dt) a.hist[k] = z;
+    for (int k = t0; k < a.ntiles; k += dt) a.tiles[k] = 0;
+    for (int k = t0; k < 6 * a.nbox; k += dt) a.bb[k] = (k % 6) < 3 ? 0x7fffffff : (int)0x80000000;  // min, max
+    if (t0 == 0) *a.stale = -1;
 }
 
 __global__ void bbox_kernel(const float4 *__restrict__ pos, const float *__restrict__ h, int n,
@@ -98,13 +116,6 @@ __global__ void bbox_kernel(const float4 *__restrict__ pos, const float *__restr
 }
 
 // batch: one box per instance (6 ordered ints each), warp-combined atomics
-__global__ void bbox_batch_init_kernel(int *bb, int n_inst)
-{
-    pdl_sync();
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 6 * n_inst; k += gridDim.x * blockDim.x)
-        bb[k] = (k % 6) < 3 ? 0x7fffffff : (int)0x80000000;
-}
-
 __global__ void bbox_batch_kernel(const float4 *__restrict__ pos, const float *__restrict__ h,
                                   const int *__restrict__ inst, int n, int *bb, int *err)
 {
@@ -182,14 +193,15 @@ __global__ void morton_kernel(const float4 *__restrict__ pos, const int *__restr
 }
 
 // ------------------------------------------------------------- radix sort
-// Stable LSD radix sort of (key, index) with 8-bit digits.  Few particles
-// share the key's top 32 bits (a cell of 2^-10 of the box per axis), so four
-// passes sort by bits 32..63 and a fix-up pass orders each run of equal top
-// bits by its low 32 bits; if some run is longer than kFixRun, eight passes
-// over the whole word follow (they return at once otherwise).  Two
-// more passes on the instance id in a batch.  The digit counts of
-// every pass are taken in one histogram pass up front (the multiset of keys
-// does not change between passes).  Each pass is then one kernel: tiles are
+// Stable LSD radix sort of (key, index) with 8-bit digits, of keys that are not
+// in order already (a state given in curve order, as the adjoint's, leaves all
+// passes at once).  Few particles share the key's top 32 bits (a cell of 2^-10
+// of the box per axis), so four passes sort by bits 32..63 and a fix-up pass
+// orders each run of equal top bits by its low 32 bits; if some run is longer
+// than kFixRun, eight passes over the whole word follow (they return at once
+// otherwise).  Two more passes on the instance id in a batch.  The digit counts
+// are taken in one histogram pass up front (the multiset of keys does not change
+// between passes).  Each pass is then one kernel: tiles are
 // numbered in launch order by an atomic counter, each ranks its keys (warp
 // match + per-warp counts, in input order, so the sort is stable), publishes
 // its per-digit counts and adds up its predecessors' counts by looking back
@@ -227,34 +239,53 @@ __device__ __forceinline__ uint32_t block_scan_256(uint32_t v, uint32_t &excl, u
     return total;
 }
 
-// digit counts of all passes: ghist[p][d] for the 8 key digits and, with
-// inst, the 2 instance-id digits.  Each thread counts RS_GE consecutive
+// Digit counts ghist[p][d] of the passes on the key digits 4..7 and, with inst,
+// the 2 instance-id digits (p = 8, 9); LOW: of the key digits 0..3, which only
+// the rare passes over all 64 bits need, so that the step's sort does not pay
+// for their scattered counts.  The first also finds whether the (instance, key)
+// pairs are in order already.  Each thread counts RS_GE consecutive
 // keys, adding runs of one digit with one shared atomic: the keys are nearly
 // in curve order, so the high digits come in long runs, and a run that spans
 // the whole warp is added once for the warp.  Four blocks per SM: each adds
 // its shared counts to ghist once, which keeps the global atomics few.
 constexpr int RS_GE = 8;
+template <bool LOW>
 __global__ void __launch_bounds__(256) rs_ghist_kernel(const uint64_t *__restrict__ keys,
                                                        const int *__restrict__ inst, int n,
-                                                       uint32_t *ghist)
+                                                       uint32_t *ghist, int *flags)
 {
     pdl_sync();
-    __shared__ uint32_t h[10][256];
-    for (int k = threadIdx.x; k < 10 * 256; k += 256) (&h[0][0])[k] = 0;
+    if (LOW && flags[RF_FULL] == 0) return;
+    constexpr int NP = LOW ? 4 : 6, P0 = LOW ? 0 : 4;
+    __shared__ uint32_t h[NP][256];
+    for (int k = threadIdx.x; k < NP * 256; k += 256) (&h[0][0])[k] = 0;
     __syncthreads();
-    const int np = inst ? 10 : 8;
+    const int np = LOW || !inst ? 4 : 6;
+    bool order = true;
     for (int b = blockIdx.x * 256 * RS_GE; b < n; b += gridDim.x * 256 * RS_GE) {
         const int s0 = b + threadIdx.x * RS_GE;
-        uint32_t cur[10], cnt[10];
+        uint32_t cur[NP], cnt[NP];
 #pragma unroll
-        for (int p = 0; p < 10; ++p) { cur[p] = 0; cnt[p] = 0; }
+        for (int p = 0; p < NP; ++p) { cur[p] = 0; cnt[p] = 0; }
+        uint64_t last = 0;  // the key before, and its instance
+        int ilast = 0;
+        if (!LOW && s0 > 0 && s0 < n) {
+            last = keys[s0 - 1];
+            ilast = np > 4 ? inst[s0 - 1] : 0;
+        }
         for (int e = 0; e < RS_GE && s0 + e < n; ++e) {
-            const uint64_t key = keys[s0 + e];
-            const uint32_t iv = inst ? (uint32_t)inst[s0 + e] : 0u;
+            const uint64_t k64 = keys[s0 + e];
+            const uint32_t key = (uint32_t)(k64 >> (8 * P0));
+            const int iv = np > 4 ? inst[s0 + e] : 0;
+            if (!LOW) {
+                order = order && (iv > ilast || (iv == ilast && k64 >= last));
+                last = k64;
+                ilast = iv;
+            }
 #pragma unroll
-            for (int p = 0; p < 10; ++p) {
+            for (int p = 0; p < NP; ++p) {
                 if (p >= np) break;
-                const uint32_t d = p < 8 ? (uint32_t)((key >> (8 * p)) & 255u) : (iv >> (8 * (p - 8))) & 255u;
+                const uint32_t d = p < 4 ? (key >> (8 * p)) & 255u : ((uint32_t)iv >> (8 * (p - 4))) & 255u;
                 if (cnt[p] != 0 && d != cur[p]) {
                     atomicAdd(&h[p][cur[p]], cnt[p]);
                     cnt[p] = 0;
@@ -264,7 +295,7 @@ __global__ void __launch_bounds__(256) rs_ghist_kernel(const uint64_t *__restric
             }
         }
 #pragma unroll
-        for (int p = 0; p < 10; ++p) {
+        for (int p = 0; p < NP; ++p) {
             if (p >= np) break;
             const uint32_t c0 = __shfl_sync(0xffffffffu, cur[p], 0);
             if (__all_sync(0xffffffffu, cnt[p] == 0 || cur[p] == c0)) {
@@ -275,21 +306,12 @@ __global__ void __launch_bounds__(256) rs_ghist_kernel(const uint64_t *__restric
             }
         }
     }
+    if (!LOW && __any_sync(0xffffffffu, !order) && (threadIdx.x & 31) == 0) flags[RF_UNSORTED] = 1;
     __syncthreads();
     for (int k = threadIdx.x; k < np * 256; k += 256) {
         const uint32_t v = (&h[0][0])[k];
-        if (v) atomicAdd(&ghist[k], v);
+        if (v) atomicAdd(&ghist[P0 * 256 + k], v);
     }
-}
-
-// gstart[p][d] = exclusive scan of ghist[p][.]   (block p)
-__global__ void __launch_bounds__(256) rs_gscan_kernel(const uint32_t *ghist, uint32_t *gstart)
-{
-    pdl_sync();
-    __shared__ uint32_t ws[8];
-    uint32_t ex;
-    block_scan_256(ghist[blockIdx.x * 256 + threadIdx.x], ex, ws);
-    gstart[blockIdx.x * 256 + threadIdx.x] = ex;
 }
 
 // One pass: warp w of a tile owns the contiguous keys [w * 256, (w + 1) * 256)
@@ -300,8 +322,8 @@ __global__ void __launch_bounds__(256) rs_gscan_kernel(const uint32_t *ghist, ui
 __global__ void __launch_bounds__(RS_T, 4) rs_onesweep_kernel(
     const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint64_t *__restrict__ kout,
     uint32_t *__restrict__ vout, const int *__restrict__ inst, int n, int shift,
-    const uint32_t *__restrict__ gstart, uint32_t *status, int *tile_counter, int *err,
-    const int *gate, int spin_cap)
+    const uint32_t *__restrict__ ghist, uint32_t *status, int *tile_counter, int *err,
+    const int *gate, const int *unsorted, int spin_cap)
 {
     pdl_sync();
     if (gate && *gate == 0) return;  // a pass of the full sort that is not needed
@@ -314,12 +336,16 @@ __global__ void __launch_bounds__(RS_T, 4) rs_onesweep_kernel(
     __shared__ uint32_t sval[RS_TILE];
     __shared__ uint8_t sdig[RS_TILE];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    if (tid == 0) s_tile = atomicAdd(tile_counter, 1);
+    if (tid == 0) {  // the flag's latency beside the counter's
+        const int t = atomicAdd(tile_counter, 1), u = unsorted ? *unsorted : 1;
+        s_tile = u ? t : -1;
+    }
     uint32_t *flat = &wcnt[0][0];
 #pragma unroll
     for (int k = 0; k < 8; ++k) flat[k * 256 + tid] = 0;
     __syncthreads();
     const int tile = s_tile;
+    if (tile < 0) return;  // the keys are in order already
     const uint32_t lt = (1u << lane) - 1u;
     const int tile0 = tile * RS_TILE;
     const int wbase = tile0 + w * (RS_TILE / 8);
@@ -350,6 +376,7 @@ __global__ void __launch_bounds__(RS_T, 4) rs_onesweep_kernel(
     __syncthreads();
     uint32_t cnt;  // keys of digit tid in this tile
     {
+        const uint32_t gh = ghist[tid];
         uint32_t acc = 0;
 #pragma unroll
         for (int ww = 0; ww < 8; ++ww) {
@@ -361,6 +388,8 @@ __global__ void __launch_bounds__(RS_T, 4) rs_onesweep_kernel(
         uint32_t ex;
         block_scan_256(acc, ex, ws);  // digit starts inside the sorted tile
         tstart[tid] = ex;
+        block_scan_256(gh, ex, ws);  // digit starts in the sorted array
+        gbase[tid] = ex;
     }
     // publish this tile's count of digit tid, then add up the predecessors'
     volatile uint32_t *st = status;
@@ -392,7 +421,7 @@ __global__ void __launch_bounds__(RS_T, 4) rs_onesweep_kernel(
         }
     }
     if (tile > 0) st[(size_t)tile * 256 + tid] = RS_INC | (excl + cnt);
-    gbase[tid] = gstart[tid] + excl;
+    gbase[tid] += excl;
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < RS_I; ++r) {
@@ -420,9 +449,10 @@ __global__ void __launch_bounds__(RS_T, 4) rs_onesweep_kernel(
 // that are not at a run's start read only the top bits of their neighbours,
 // which the sort inside a run does not change.
 constexpr int kFixRun = 32;
-__global__ void rs_fixup_kernel(uint64_t *keys, uint32_t *vals, int n, int *full)
+__global__ void rs_fixup_kernel(uint64_t *keys, uint32_t *vals, int n, int *full, const int *gate)
 {
     pdl_sync();
+    if (*gate == 0) return;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
         const uint64_t top = keys[s] >> 32;
         if (s > 0 && (keys[s - 1] >> 32) == top) continue;        // inside a run
@@ -1083,6 +1113,19 @@ static int grid_for(const Ctx &c, int64_t n, int block)
         if (e_ != cudaSuccess) return e_;           \
     } while (0)
 
+__global__ void clear_kernel(Clear z)
+{
+    pdl_sync();
+    for (int a = 0; a < 3; ++a)
+        for (int k = threadIdx.x; k < z.n[a]; k += blockDim.x) z.p[a][k] = 0;
+}
+
+cudaError_t clear_words(const Clear &z, cudaStream_t st)
+{
+    launch(clear_kernel, 1, 256, 0, st, z);
+    return cudaGetLastError();
+}
+
 cudaError_t instance_map(Ctx &c, const int64_t *d_offsets, int n_inst, int n, cudaStream_t st)
 {
     int *bad = c.d_sizes + SZ_BAD_OFFSETS;
@@ -1108,7 +1151,8 @@ cudaError_t refit_tree(Ctx &c, const sph_state &s, cudaStream_t st)
 
 int tree_launches(int64_t n, bool full)
 {
-    // box (2), keys, sort, gather (and copy back), chop flags, scans, counts, nodes (2), bounds
+    // start, box, keys, sort (digit counts, twice), gather (and copy back), chop flags, scans,
+    // counts, nodes (2), bounds
     const int sort = n <= kRankSort ? 1 : 2 + 4 + 1 + 8;
     const int scans = (n <= kScanOne ? 1 : 3) + (kLevels * (int64_t)div_up(n, kChopBlock) <= kScanOne ? 1 : 3);
     return 3 + sort + 2 + (full ? 1 : 0) + scans + 4;
@@ -1129,11 +1173,26 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
     float4 *pos_in = kicked ? c.tmp4[0] : pos;
     const float *h_in = kicked ? c.tmp1[0] : s.h;
     // 1. bounding box (per instance in a batch) and input checks
+    const bool radix = n > kRankSort;
+    const int ntiles = div_up(n, RS_TILE);
+    const int nslot = 4 + 8 + (batch ? 2 : 0);
+    int *flags = c.rs_tiles + kRsSlots;
+    BuildInit init{};
+    init.bb = bb;
+    init.nbox = batch ? batch->n_inst : 1;
+    init.stale = t.rec_ctl + 1;
+    if (radix) {
+        init.hist = (uint4 *)c.rs_ghist;
+        init.nhist = 10 * 256 / 4;
+        init.status = (uint4 *)c.rs_status;
+        init.nstatus = 256 / 4 * ntiles * nslot;
+        init.tiles = c.rs_tiles;
+        init.ntiles = kRsSlots + kRsFlags;
+    }
+    launch(build_init_kernel, radix ? grid_for(c, init.nstatus, 256) : div_up(6 * init.nbox, 256), 256, 0, st, init);
     if (batch) {
-        launch(bbox_batch_init_kernel, div_up(6 * batch->n_inst, 256), 256, 0, st, bb, batch->n_inst);
         launch(bbox_batch_kernel, grid_for(c, n, 256), 256, 0, st, pos_in, h_in, inst, n, bb, c.d_err);
     } else {
-        launch(bbox_init_kernel, 1, 32, 0, st, bb);
         launch(bbox_kernel, grid_for(c, n, 256), 256, 0, st, pos_in, h_in, n, bb, c.d_err);
     }
     // 2. keys
@@ -1144,42 +1203,39 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
     //    instance back on its own slots
     uint64_t *kin = s.keys, *kout = c.keys_alt;
     uint32_t *vin = c.idx_a, *vout = c.idx_b;
-    if (n <= kRankSort) {
+    if (!radix) {
         const int grid = div_up(n, kRankE);
         if (batch) launch(rank_sort_kernel<true>, grid, kRankE * kRankP, 0, st, kin, inst, n, kout, vout);
         else launch(rank_sort_kernel<false>, grid, kRankE * kRankP, 0, st, kin, nullptr, n, kout, vout);
         std::swap(kin, kout);
         std::swap(vin, vout);
     } else {
-        const int ntiles = div_up(n, RS_TILE);
-        const int ndigit = batch ? 10 : 8;  // digits 0..7 of the key, 8..9 of the instance id
-        const int nslot = 4 + 8 + (batch ? 2 : 0);
-        int *full = c.rs_tiles + kRsSlots;  // the fix-up found a long run: sort all 64 bits
-        // digit counts of all passes, their scans, fresh look-back words, tile counters, flag
-        SPH_TRY(cudaMemsetAsync(c.rs_ghist, 0, sizeof(uint32_t) * 10 * 256, st));
-        SPH_TRY(cudaMemsetAsync(c.rs_tiles, 0, sizeof(int) * (kRsSlots + 1), st));
-        SPH_TRY(cudaMemsetAsync(c.rs_status, 0, sizeof(uint32_t) * 256 * (size_t)ntiles * nslot, st));
+        // digits 0..7 of the key, 8..9 of the instance id
+        // Nothing moves if the keys are in order already (a state given in curve
+        // order, as the adjoint's): an even number of passes leaves the pairs
+        // where they were.
+        int *full = flags + RF_FULL, *unsorted = flags + RF_UNSORTED;
         const int gh_grid = (int)std::max<int64_t>(1, std::min<int64_t>(div_up(n, 256 * RS_GE), 4 * (int64_t)c.num_sms));
-        launch(rs_ghist_kernel, gh_grid, 256, 0, st, kin, inst, n, c.rs_ghist);
-        launch(rs_gscan_kernel, ndigit, 256, 0, st, c.rs_ghist, c.rs_gstart);
+        launch(rs_ghist_kernel<false>, gh_grid, 256, 0, st, kin, inst, n, c.rs_ghist, flags);
         int slot = 0;
-        auto pass = [&](int digit, const int *gate) {
+        auto pass = [&](int digit, const int *gate, const int *unsorted) {
             const int *dinst = digit >= 8 ? inst : nullptr;
             const int shift = digit >= 8 ? 8 * (digit - 8) : 8 * digit;
             launch(rs_onesweep_kernel, ntiles, RS_T, 0, st, kin, vin, kout, vout, dinst, n, shift,
-                                                        c.rs_gstart + 256 * digit,
+                                                        c.rs_ghist + 256 * digit,
                                                         c.rs_status + (size_t)256 * ntiles * slot,
-                                                        c.rs_tiles + slot, c.d_err, gate, RS_SPIN);
+                                                        c.rs_tiles + slot, c.d_err, gate, unsorted, RS_SPIN);
             ++slot;
             std::swap(kin, kout);  // a gated pass that returns moves nothing, but
             std::swap(vin, vout);  // the gated passes come in an even number
         };
-        for (int digit = 4; digit < 8; ++digit) pass(digit, nullptr);
-        launch(rs_fixup_kernel, grid_for(c, n, 256), 256, 0, st, kin, vin, n, full);
-        for (int digit = 0; digit < 8; ++digit) pass(digit, full);
+        for (int digit = 4; digit < 8; ++digit) pass(digit, nullptr, unsorted);
+        launch(rs_fixup_kernel, grid_for(c, n, 256), 256, 0, st, kin, vin, n, full, unsorted);
+        launch(rs_ghist_kernel<true>, gh_grid, 256, 0, st, kin, inst, n, c.rs_ghist, flags);
+        for (int digit = 0; digit < 8; ++digit) pass(digit, full, nullptr);
         if (batch) {
-            pass(8, nullptr);
-            pass(9, nullptr);
+            pass(8, nullptr, unsorted);
+            pass(9, nullptr, unsorted);
         }
     }
     // the sorted (key, slot) pairs are in (kin, vin)
@@ -1218,8 +1274,6 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
         launch(gather_kernel, grid_for(c, n, 256), 256, 0, st, g, n);
         launch(copy_back_kernel, grid_for(c, n, 256), 256, 0, st, g, n);
     }
-    // recorded leaf ranges refer to the previous tree: mark them invalid
-    SPH_TRY(cudaMemsetAsync(t.rec_ctl + 1, 0xff, sizeof(int), st));
     // 5. chop: tree (n_leaf) and groups (n_group)
     if (n < kCfTile * c.num_sms)
         launch(chop_flags_kernel<kCfSmall>, grid_for(c, n, kCfSmall), 256, 0, st, s.keys, inst, n, p.n_leaf,
@@ -1279,7 +1333,7 @@ cudaError_t sort_lookback_probe(Ctx &c, int spin_cap, cudaStream_t st)
     SPH_TRY(cudaMemsetAsync(c.rs_status, 0, sizeof(uint32_t) * 256 * 2, st));
     launch(set_int_kernel, 1, 1, 0, st, c.rs_tiles, 1);  // the block draws tile 1
     launch(rs_onesweep_kernel, 1, RS_T, 0, st, c.keys_alt, c.idx_a, c.keys_alt, c.idx_b, nullptr, RS_TILE,
-                                          0, c.rs_gstart, c.rs_status, c.rs_tiles, c.d_err, nullptr,
+                                          0, c.rs_ghist, c.rs_status, c.rs_tiles, c.d_err, nullptr, nullptr,
                                           spin_cap);
     return cudaGetLastError();
 }
