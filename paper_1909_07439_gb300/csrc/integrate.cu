@@ -93,23 +93,41 @@ __global__ void dt_batch_init_kernel(int *dtmin, int n_inst)
         dtmin[k] = 0x7f800000;  // +inf
 }
 
-__global__ void dt_batch_kernel(const float *__restrict__ h, const float *__restrict__ vs,
-                                const int *__restrict__ inst, int n, int *dtmin)
+// a warp takes a contiguous range of particles and combines them while they
+// stay in one instance (an atomic per 32 particles: 37 us for 1.6 M particles in
+// 48 instances, so 16 us)
+__global__ void __launch_bounds__(256) dt_batch_kernel(const float *__restrict__ h, const float *__restrict__ vs,
+                                                       const int *__restrict__ inst, int n, int per, int *dtmin)
 {
     pdl_sync();
-    for (int i0 = blockIdx.x * blockDim.x; i0 < n; i0 += gridDim.x * blockDim.x) {
-        int i = i0 + threadIdx.x;
-        bool in = i < n;
-        float m = in ? h[i] / vs[i] : INFINITY;
-        int k = in ? inst[i] : -1;
-        int k0 = __shfl_sync(0xffffffffu, k, 0);
-        if (__all_sync(0xffffffffu, k == k0)) {
-            for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if ((threadIdx.x & 31) == 0 && k0 >= 0) atomicMin(dtmin + k0, __float_as_int(m));
+    const int lane = threadIdx.x & 31, warp = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int64_t s0 = (int64_t)warp * per;
+    const int s1 = (int)min((int64_t)n, s0 + per);
+    int kc = -1;
+    float m = INFINITY;
+    auto flush = [&]() {
+        for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (lane == 0) atomicMin(dtmin + kc, __float_as_int(m));
+        m = INFINITY;
+    };
+    for (int64_t s = s0; s < s1; s += 32) {
+        const int i = (int)s + lane;
+        const bool in = i < s1;
+        const float v = in ? h[i] / vs[i] : INFINITY;
+        const int k = in ? inst[i] : -1, k0 = __shfl_sync(0xffffffffu, k, 0);
+        const bool one = __all_sync(0xffffffffu, !in || k == k0);
+        if (kc >= 0 && !(one && k0 == kc)) {
+            flush();
+            kc = -1;
+        }
+        if (one) {
+            kc = k0;
+            m = fminf(m, v);
         } else if (in) {
-            atomicMin(dtmin + k, __float_as_int(m));
+            atomicMin(dtmin + k, __float_as_int(v));
         }
     }
+    if (kc >= 0) flush();
 }
 
 __global__ void dt_batch_final_kernel(const int *dtmin, int n_inst, float c_cour, float *d_dt)
@@ -360,7 +378,8 @@ cudaError_t courant_dt(Ctx &c, const sph_state &s, const sph_params &p, float *d
     if (batch) {
         const int ni = batch->n_inst;
         launch(dt_batch_init_kernel, div_up(ni, 256), 256, 0, st, c.dtmin_inst, ni);
-        launch(dt_batch_kernel, grid_n(c, n, 256), 256, 0, st, s.h, s.vsigmax, c.inst, n, c.dtmin_inst);
+        const int per = 32 * std::max(1, div_up(n, 32 * 8 * 4 * c.num_sms));  // particles a warp
+        launch(dt_batch_kernel, div_up(n, 8 * per), 256, 0, st, s.h, s.vsigmax, c.inst, n, per, c.dtmin_inst);
         launch(dt_batch_final_kernel, div_up(ni, 256), 256, 0, st, c.dtmin_inst, ni, p.c_cour, d_dt);
         return cudaGetLastError();
     }
