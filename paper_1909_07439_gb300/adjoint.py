@@ -5,9 +5,9 @@ density solve, force pass) returning h, rho, Omega and acc = (a, du/dt) in
 the caller's particle order; its backward takes arbitrary cotangents of those
 outputs and returns dL/dx, dL/d(v, u) and dL/dalpha_AV from the library's
 adjoint kernels (sph_force_bwd, then sph_density_bwd through the h-rho
-fixed point by the implicit-function theorem).  The backward rebuilds the
-evaluation's tree and neighbour lists (deterministic kernels: the same neighbour
-sets), so the context may be used for other work in between.
+fixed point by the implicit-function theorem), taken at the forward's own h, rho
+and Omega.  The backward rebuilds the tree and the neighbour lists, so the context
+may be used for other work in between.
 
 ``rollout_loss(ctx, pos, velu, h, alpha, ...)`` returns the scalar loss
 (mean squared density of probe particles after n_steps leapfrog steps) as a
@@ -60,29 +60,33 @@ class _Evaluate(torch.autograd.Function):
         for f in ("h", "rho", "omega", "acc"):
             a = getattr(s, f)[:n]
             out.append(torch.empty_like(a).index_copy_(0, perm, a))   # curve order -> caller order
-        # the inputs too: a change of theirs before the backward pass is an error
-        fctx.save_for_backward(pos, velu, h0, alpha, perm, s.pos, s.vel, s.h)
+        # the inputs too: a change of theirs before the backward pass is an error;
+        # the outputs' values in curve order and the order (16 bytes per particle)
+        # are copies, so that the caller may change the outputs
+        fctx.save_for_backward(pos, velu, h0, alpha, s.perm, s.h, s.rho, s.omega)
         fctx.handle, fctx.p = handle, p
         return tuple(out)
 
     @staticmethod
     def backward(fctx, gh, grho, gom, gacc):
-        pos, velu, h0, alpha, perm, spos, svel, sh = fctx.saved_tensors
+        pos, velu, h0, alpha, perm, h, rho, omega = fctx.saved_tensors
         handle, p = fctx.handle, fctx.p
-        # The tree and the lists of the state in the forward's curve order (the
-        # sort is the identity) at its converged h, where the density pass needs
-        # one sweep and no batch leaves the list pad; the adjoint passes read
-        # nothing else of a force pass.  A fixed number of Newton updates starts
-        # from h0 again.  (With the whole evaluation repeated from h0 and its
-        # arrays zeroed first, forward and backward of 30011 particles took 3.05 ms;
-        # so 2.25 ms.)
         n, dev = pos.shape[0], pos.device
-        if p.density_iters > 0:
-            s = _state(pos, velu, h0)
-        else:
-            s = _state(spos[:n], svel[:n], sh[:n])
+        perm = perm.long()
+        # The forward's tree and the lists of its h, rho and Omega, at which it is
+        # differentiated: the state in the forward's curve order (the sort is the
+        # identity), one sweep of the density pass that accepts any h (a Newton
+        # step is at most h), so that no batch leaves the list pad, and the
+        # forward's rho and Omega in place of that sweep's.  The adjoint passes
+        # read nothing of a force pass.
+        s = DeviceState(n, device=dev, zero=False)
+        s.pos, s.vel = pos.detach().index_select(0, perm), velu.detach().index_select(0, perm)
+        s.h.copy_(h)
+        q = _params(p, p.alpha_av)
+        q.density_iters, q.h_tol = 0, 4.0
         native.sph_build_tree(handle, s.c, p)
-        native.sph_density(handle, s.c, p)
+        native.sph_density(handle, s.c, q)
+        s.rho, s.omega = rho, omega
 
         def to_curve(g, shape):
             return (torch.zeros(shape, dtype=torch.float32, device=dev) if g is None
