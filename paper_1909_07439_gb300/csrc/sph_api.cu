@@ -427,6 +427,7 @@ sph_status sph_create(sph_ctx **out, int64_t max_n, int device)
     A(dalloc(t.lv_tree, n));
     A(dalloc(t.lv_grp, n));
     A(dalloc(t.blk_cnt, (size_t)kLevels * nbchop));
+    A(dalloc(t.blk_off, (size_t)kLevels * nbchop));  // more than max_n entries below 22 particles
     A(dalloc(c.rec, 2 * n));
     A(dalloc(c.prop, n));
     A(dalloc(c.frec, 3 * n));
@@ -471,7 +472,7 @@ void sph_destroy(sph_ctx *h)
                     c.tree.node_first, c.tree.node_count, c.tree.node_level, c.tree.node_child,
                     c.tree.node_nchild, c.tree.node_parent, c.tree.node_arrive, c.tree.node_lo,
                     c.tree.node_hi, c.tree.node_ref, c.tree.grp_ref,
-                    c.tree.grp_lo, c.tree.grp_hi, c.tree.lv_tree, c.tree.lv_grp, c.tree.blk_cnt,
+                    c.tree.grp_lo, c.tree.grp_hi, c.tree.lv_tree, c.tree.lv_grp, c.tree.blk_cnt, c.tree.blk_off,
                     c.nl_idx, c.nl_len, c.fallback,
                     c.tree.rec_ctl, c.tree.rec_bad,
                     c.rec, c.prop, c.frec, c.vhalf, c.active, c.g_com, c.g_q0, c.g_q1, c.inst, c.bbox_inst,

@@ -89,7 +89,8 @@ struct Tree {
     int *rec_bad = nullptr;
     // chop scratch
     int *lv_tree = nullptr, *lv_grp = nullptr;
-    int *blk_cnt = nullptr;      // [kLevels][nb]
+    int *blk_cnt = nullptr;      // [kLevels][nb] nodes per level and block of slots
+    int *blk_off = nullptr;      // [kLevels][nb] their exclusive scan
 };
 
 // a batch of independent instances packed back to back

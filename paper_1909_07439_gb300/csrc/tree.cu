@@ -1341,12 +1341,11 @@ cudaError_t build_tree(Ctx &c, const sph_state &s, const sph_params &p, bool ful
     SPH_TRY(scan_mode(c, t.lv_grp, nullptr, n, 1, c.d_sizes + SZ_GROUPS, st, t.grp_ref));
     // nodes
     int nb = div_up(n, kChopBlock);
-    int *blk_off = (int *)c.tmp1[2];
     int *ntotal = c.d_sizes + 2;
     launch(chop_count_kernel, nb, 256, 0, st, t.lv_tree, n, t.blk_cnt, nb);
-    SPH_TRY(scan_mode(c, t.blk_cnt, blk_off, kLevels * nb, 0, ntotal, st));
-    launch(chop_write_kernel, nb, 256, 0, st, t.lv_tree, n, blk_off, nb, ntotal, t, c.d_sizes, c.d_err);
-    launch(node_finish_kernel, grid_for(c, node_cap_for(t, n), 256), 256, 0, st, s.keys, inst, n, p.n_leaf, blk_off,
+    SPH_TRY(scan_mode(c, t.blk_cnt, t.blk_off, kLevels * nb, 0, ntotal, st));
+    launch(chop_write_kernel, nb, 256, 0, st, t.lv_tree, n, t.blk_off, nb, ntotal, t, c.d_sizes, c.d_err);
+    launch(node_finish_kernel, grid_for(c, node_cap_for(t, n), 256), 256, 0, st, s.keys, inst, n, p.n_leaf, t.blk_off,
                                                                               nb, t, c.d_sizes);
     SPH_TRY(launch_bounds(c, s, 0, nullptr, st));
     return cudaGetLastError();
