@@ -86,8 +86,8 @@ __device__ __forceinline__ float seg_sum(float v, int L)
 
 // Sums of one pair at smoothing length 1/hinv (kernel K, whose f and f'
 // vanish beyond its support):
-//   s0 += m_j f(q) / F0, s1 += m_j (3 f + q f') / F1, s2 += m_j vd f' / r
-// (h^3 rho = C F0 s0, -h^4 d(rho)/dh = C F1 s1, Eq. 3 numerator x h^4 / C = s2).
+//   s0 += m_j f(q), s1 += m_j (3 f + q f'), s2 += m_j vd f' / r
+// (h^3 rho = C s0, -h^4 d(rho)/dh = C s1, Eq. 3 numerator x h^4 / C = s2).
 template <int K, bool VD = true>
 __device__ __forceinline__ void pair_sums(float r2, float mj, float vd, float hinv, float &s0,
                                           float &s1, float &s2)
@@ -95,10 +95,10 @@ __device__ __forceinline__ void pair_sums(float r2, float mj, float vd, float hi
     // r = 0 (the particle itself, or a padding entry) gives q = 0 and vd = 0
     const float rinv = rsqrt_normal(fmaxf(r2, 1e-30f));
     const float q = r2 * rinv * hinv;
-    float f, g, df;
-    SphKernel<K>::sums(q, f, g, df);
+    float f, df;
+    SphKernel<K>::f_df(q, f, df);
     s0 += mj * f;
-    s1 += mj * g;
+    s1 += mj * (3.f * f + q * df);
     if (VD) s2 += mj * vd * df * rinv;
 }
 
@@ -294,8 +294,8 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
                             entry(p1, v1, b1 ? p1.w : 0.f, b1);
                         }
                     }
-                    s0 = SphKernel<K>::F0 * seg_sum(s0, L);
-                    s1 = SphKernel<K>::F1 * seg_sum(s1, L);
+                    s0 = seg_sum(s0, L);
+                    s1 = seg_sum(s1, L);
                     s2 = seg_sum(s2, L);
                     const float cf = seg_sum((float)cnt, L);
                     if (sub == 0 && on) {
@@ -505,8 +505,8 @@ __global__ void __launch_bounds__(kDensWarps * 32, 4) density_walk_kernel(DensAr
                 } else {
                     list_sums();
                 }
-                s0 = SphKernel<K>::F0 * seg_sum(s0, L);
-                s1 = SphKernel<K>::F1 * seg_sum(s1, L);
+                s0 = seg_sum(s0, L);
+                s1 = seg_sum(s1, L);
                 s2 = seg_sum(s2, L);
                 const float cf = seg_sum((float)cnt, L);
                 if (sub == 0 && on) {

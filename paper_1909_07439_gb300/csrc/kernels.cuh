@@ -11,9 +11,7 @@
 //   K = 2  Wendland C6, R = 2, C = 1365/(512 pi)
 //          f = s^8 (4 q^3 + 25/4 q^2 + 4 q + 1), s = (1 - q/2)+
 // (x)+ = max(x, 0): each form is branch-free and vanishes beyond the support.
-// Members: f_df(q) -> f, f'; df(q) = f'; d2f(q) = f''; sums(q) -> f / F0,
-// (3 f + q f') / F1, f', the density sums with constant factors left to their
-// totals; and, in the variable
+// Members: f_df(q) -> f, f'; df(q) = f'; d2f(q) = f''; and, in the variable
 // p = r / (R h) = r rsqrt((R h)^2) that the force pass evaluates,
 // f'(R p) = G g_p(p) with the constant G kept apart so that it folds into a
 // per-particle factor.
@@ -32,9 +30,8 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 
 // 1 / sqrt(x) of a normal number in one instruction: rsqrtf spends three more on
 // scaling subnormal arguments, which the pair loops exclude beforehand (and their
-// kernels are bound by instruction issue and L1 together: with this and the M4
-// sums below the 128^3 density stage takes 586 instead of 608 us, force 719
-// instead of 735 us, gravity of 256 k particles 1650 instead of 1719 us)
+// kernels are bound by instruction issue and L1 together: the 128^3 force stage
+// 735 -> 719 us, gravity of 256 k particles 1719 -> 1650)
 __device__ __forceinline__ float rsqrt_normal(float x)
 {
     float r;
@@ -49,6 +46,9 @@ template <>
 struct SphKernel<0> {
     static constexpr float R = 2.f;
     static constexpr float C = 0.318309886183790671538f;
+    // Each branch by its own polynomial.  As differences of one-sided powers,
+    // t^3 / 4 - s^3 and so on with s = (1 - q)+, the sums need no select (0.3 % of a
+    // step), but f' near 0 loses its digits: 4e-4 of drho/dt at q = 2e-4.
     __device__ static __forceinline__ void f_df(float q, float &f, float &df)
     {
         const float fi = 1.f + q * q * (-1.5f + 0.75f * q);
@@ -58,17 +58,6 @@ struct SphKernel<0> {
         const bool in = q < 1.f;
         f = in ? fi : 0.25f * t2 * t;
         df = in ? dfi : -0.75f * t2;
-    }
-    // with t = (2 - q)+, s = (1 - q)+: f = t^3 / 4 - s^3, f' = 3 s^2 - 3/4 t^2,
-    // 3 f + q f' = 3/2 (t^2 (t - 1) + s^2 (2 - 4 s))
-    static constexpr float F0 = 0.25f, F1 = 1.5f;
-    __device__ static __forceinline__ void sums(float q, float &f, float &g, float &df)
-    {
-        const float t = fmaxf(2.f - q, 0.f), s = fmaxf(1.f - q, 0.f);
-        const float t2 = t * t, s2 = s * s;
-        f = fmaf(-4.f, s2 * s, t2 * t);
-        g = fmaf(s2, fmaf(-4.f, s, 2.f), t2 * (t - 1.f));
-        df = fmaf(3.f, s2, -0.75f * t2);
     }
     __device__ static __forceinline__ float d2f(float q)
     {
@@ -101,12 +90,6 @@ struct SphKernel<1> {
         const float a4 = a2 * a2, b4 = b2 * b2, c4 = c2 * c2;
         f = fmaf(15.f * c4, c, fmaf(-6.f * b4, b, a4 * a));
         df = -5.f * fmaf(15.f, c4, fmaf(-6.f, b4, a4));
-    }
-    static constexpr float F0 = 1.f, F1 = 1.f;
-    __device__ static __forceinline__ void sums(float q, float &f, float &g, float &df)
-    {
-        f_df(q, f, df);
-        g = fmaf(q, df, 3.f * f);
     }
     __device__ static __forceinline__ float df(float q)
     {
@@ -142,12 +125,6 @@ struct SphKernel<2> {
         const float P = fmaf(fmaf(fmaf(4.f, q, 6.25f), q, 4.f), q, 1.f);
         f = s7 * s * P;
         df = -5.5f * q * s7 * fmaf(fmaf(4.f, q, 3.5f), q, 1.f);
-    }
-    static constexpr float F0 = 1.f, F1 = 1.f;
-    __device__ static __forceinline__ void sums(float q, float &f, float &g, float &df)
-    {
-        f_df(q, f, df);
-        g = fmaf(q, df, 3.f * f);
     }
     __device__ static __forceinline__ float df(float q)
     {
