@@ -50,7 +50,9 @@ struct DensArgs {
     const float4 *vel;
     const float4 *rec;  // pos, vel side by side
     float *h, *rho, *omega, *drhodt;
-    float *h_try;  // h that a batch handed over had reached (scratch)
+    // where the targets of a batch handed over had got to (scratch): h, its
+    // bracket and the updates done (as an int)
+    float4 *reached;
     float4 *prop;  // h, rho, 1/(rho Omega), c_s  (for the force pass)
     // the force records and their checks too (force_prep_kernel), or nullptr
     float4 *frec;
@@ -162,11 +164,12 @@ __device__ __forceinline__ void density_outputs(const DensArgs &a, int i, float 
     }
 }
 
-// hands a batch over at the h its targets reached (h of target i, in the lanes
-// of mine)
-__device__ __forceinline__ void push_fallback(const DensArgs &a, int g, int b0, int nt, bool mine, int i, float h)
+// hands a batch over where its targets got to in `it` updates (target i in the
+// lanes of mine; a converged one with its bracket closed, which keeps its h)
+__device__ __forceinline__ void push_fallback(const DensArgs &a, int g, int b0, int nt, bool mine, int i, float h,
+                                              float hlo, float hhi, int it)
 {
-    if (mine) a.h_try[i] = h;
+    if (mine) a.reached[i] = make_float4(h, hlo, hhi, __int_as_float(it));
     if ((threadIdx.x & 31) == 0) push_fallback_batch(a.fallback, a.n_fallback, g, b0, nt);
 }
 
@@ -218,7 +221,7 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
                 if (!__any_sync(0xffffffffu, on)) continue;  // no target of the batch is due
                 const int len = act ? a.nl_len[i] : 0;
                 if (__any_sync(0xffffffffu, len < 0)) {  // no list (overflow, or too many leaves)
-                    push_fallback(a, g, b0, nt, act && sub == 0, i, a.h[i]);
+                    push_fallback(a, g, b0, nt, act && sub == 0, i, a.h[i], 0.f, INFINITY, 0);
                     continue;
                 }
                 const int *__restrict__ lst = a.nl_idx + (size_t)i * a.nl_stride;
@@ -319,7 +322,7 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
                     }
                 }
                 if (__any_sync(0xffffffffu, outside)) {  // go on with walks
-                    push_fallback(a, g, b0, nt, act && sub == 0, i, h);
+                    push_fallback(a, g, b0, nt, act && sub == 0, i, h, conv ? h : hlo, conv ? h : hhi, it);
                     continue;
                 }
                 if (on && sub == 0) density_outputs<K, !VD>(a, i, h, M, s1, s2, xi, vi, VD);
@@ -338,11 +341,11 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
 }
 
 // Batches the list kernel handed over, each solved with tree walks from the h
-// it had reached there, whose first updates are the largest (a fixed number of
-// updates starts over from the starting h).  Bound by the latency of its walks:
-// a warp's next candidates are loaded while it tests the ones before, its
-// batches have 4 targets, and lists that overflow are summed while walking in
-// that sweep only.  Density stage, before (from the starting
+// it had reached there, whose first updates are the largest, with its bracket and
+// its count of updates (a fixed number of updates starts over from the starting
+// h).  Bound by the latency of its walks: a warp's next candidates are loaded
+// while it tests the ones before, its batches have 4 targets, and lists that
+// overflow are summed while walking in that sweep only.  Density stage, before (from the starting
 // h, whole batches, no prefetch, streaming for good) and now: 8192 particles
 // from a rough h (1248 batches) 262 -> 161 us, the M6 tube (76 batches past the
 // list capacity) 392 -> 323 us.  List pads of 6 and 10 % instead of 3 were no
@@ -388,15 +391,17 @@ __global__ void __launch_bounds__(kDensWarps * 32, 4) density_walk_kernel(DensAr
             }
             __syncwarp();
             const float h_in = a.h[i];
-            float h = fixed ? h_in : a.h_try[i];
+            const float4 from = fixed ? make_float4(h_in, 0.f, INFINITY, __int_as_float(0)) : a.reached[i];
+            float h = from.x;
             const float M = sm.tp[act ? t : 0].w * hf3;  // m_i hfact^3
-            float hlo = 0.f, hhi = INFINITY;
+            float hlo = from.y, hhi = from.z;
             float hw = h * (1.f + kPad);  // list radius is R hw
             bool valid = false;               // lists cover the current h
             bool streamed = false;            // batch overflowed the tile
             bool conv = !on;
-            bool final_pass = false;
-            int it = 0;
+            int it = __float_as_int(from.w);  // the same for the targets of a batch
+            bool final_pass = !fixed && it >= limit;  // the last update left the pad
+            if (final_pass && lane == 0) raise_error(a.err, SPH_ERR_NOT_CONVERGED);
             float s0, s1, s2;
             while (true) {
                 // ---- one sweep: sums at the current h of every target
@@ -855,7 +860,7 @@ cudaError_t density_solve(Ctx &c, const sph_state &s, const sph_params &p, cudaS
     a.rec = c.rec;
     a.vd = c.drhodt_in_force ? 0 : 1;
     a.h = s.h;
-    a.h_try = c.tmp1[3];  // free between tree builds
+    a.reached = c.tmp4[3];  // free between the tree build and the adjoint
     a.rho = s.rho;
     a.omega = s.omega;
     a.drhodt = s.drhodt;
