@@ -535,7 +535,7 @@ __global__ void __launch_bounds__(kDensWarps * 32, 4) density_walk_kernel(DensAr
                 }
                 __syncwarp();
             }
-            if (on && sub == 0) density_outputs<K, true>(a, i, h, M, s1, s2, sm.tp[t], sm.tv[t]);
+            if (on && sub == 0) density_outputs<K, true>(a, i, h, M, s1, s2, sm.tp[t], sm.tv[t], a.vd != 0);
             // the neighbour lists hold while no h grew beyond their pad
             if (__any_sync(0xffffffffu, on && h > a.h_in_scale * h_in) && lane == 0) {
                 atomicOr(a.rec_bad + root, 1);  // root = this group's instance
