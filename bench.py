@@ -6,7 +6,9 @@ step is one full sph_step: kick/drift, Morton-key tree build (keys, radix
 sort, permutation, chop), group walk + h-rho Newton density solve, force
 pass, closing kick and Courant step, all on the device.
 
-Prints ONE JSON line (rank 0).  ``--impl reference`` times the FP64 CPU
+Prints ONE JSON line (rank 0) to stdout, the headline with one figure of every
+other leg, and before it the whole record, with the tuner's tables, as one line to
+stderr.  ``--impl reference`` times the FP64 CPU
 oracle on a bounded sample of the same workload instead (the CPU baseline
 arm).  Multi-GPU runs are independent replicas (the step is a single problem
 and is not sharded), launched one process per GPU by torchrun.
@@ -836,6 +838,25 @@ def run_reference(args):
             "note": "FP64 brute-force CPU oracle (the reference arm); per-particle rate"}
 
 
+def headline(out):
+    """The stdout line of a record: the headline's own entries, one figure of every other leg."""
+    line = {k: out[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+                                "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config",
+                                "pair_interactions_per_s", "e2e", "gpu_launches", "stage_ms_per_step")
+            if k in out}
+    for k, names in (("clocks", ("sm_mhz", "sm_max_mhz", "reasons", "samples")),
+                     ("roofline", ("kernel", "bound", "achieved", "peak", "unit", "frac")),
+                     ("cpu_baseline", ("value", "unit", "cores", "kind")),
+                     ("batched", ("value", "batched_over_plain")),
+                     ("adjoint", ("forward_value", "forward_backward_value")),
+                     ("plummer", ("value", "ms_per_evaluation")),
+                     ("tube", ("value", "ms_per_step")),
+                     ("block", ("global_ms", "block_ms", "speedup"))):
+        if out.get(k):
+            line[k] = {n: out[k][n] for n in names if n in out[k]}
+    return line
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -863,6 +884,9 @@ def main():
     if args.warmup < 3 and args.impl == "ours":
         args.warmup = 3
     out = run_reference(args) if args.impl == "reference" else run_ours(args)
+    if out is not None and args.impl == "ours":
+        print(json.dumps(out), file=sys.stderr, flush=True)
+        out = headline(out)
     if out is not None:
         print(json.dumps(out), flush=True)
 
