@@ -59,7 +59,6 @@ struct DensArgs {
     size_t fstride;  // between the words of a record
     float alpha, gc, h_lim;
     const int2 *grp_ref;
-    const float4 *grp_lo, *grp_hi;
     const int *sizes;
     int *work, *work2;
     WalkTree tree;
@@ -871,8 +870,6 @@ cudaError_t density_solve(Ctx &c, const sph_state &s, const sph_params &p, cudaS
     a.gc = kernel_gc(p.kernel);
     a.h_lim = periodic_h_limit(p);
     a.grp_ref = c.tree.grp_ref;
-    a.grp_lo = c.tree.grp_lo;
-    a.grp_hi = c.tree.grp_hi;
     a.sizes = c.d_sizes;
     a.work = c.d_sizes + SZ_WORK;
     a.work2 = c.d_sizes + SZ_WORK2;

@@ -45,7 +45,6 @@ struct ForceArgs {
     float *vsigmax;
     float *drhodt;  // written too (Eq. 3, the pressure-work sum over m_j F_i), or nullptr
     const int2 *grp_ref;
-    const float4 *grp_lo, *grp_hi;
     const int *sizes;
     int *work, *work2;
     WalkTree tree;
@@ -671,8 +670,6 @@ cudaError_t force_pass(Ctx &c, const sph_state &s, const sph_params &p, cudaStre
     a.vsigmax = s.vsigmax;
     a.drhodt = c.drhodt_in_force ? s.drhodt : nullptr;
     a.grp_ref = c.tree.grp_ref;
-    a.grp_lo = c.tree.grp_lo;
-    a.grp_hi = c.tree.grp_hi;
     a.sizes = c.d_sizes;
     a.work = c.d_sizes + SZ_WORK;
     a.work2 = c.d_sizes + SZ_WORK2;

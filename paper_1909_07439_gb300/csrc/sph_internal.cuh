@@ -110,7 +110,7 @@ struct Ctx {
     uint32_t *idx_a = nullptr, *idx_b = nullptr;
     uint32_t *rs_ghist = nullptr;   // [10][256] digit counts of every pass
     uint32_t *rs_status = nullptr;  // [kRsSlots][ntiles][256] look-back words, one slot per pass
-    int *rs_tiles = nullptr;        // [kRsSlots] tile counters, then the flags of rs_flag
+    int *rs_tiles = nullptr;        // [kRsSlots] tile counters, then the flags RF_*
     int ntiles_cap = 0;
 
     // gather scratch
@@ -266,8 +266,6 @@ cudaError_t update_hmax(Ctx &c, const sph_state &s, const sph_params &p, cudaStr
                         const int *gate = nullptr);
 // c.rec from the state's pos and vel (build_tree writes it too)
 cudaError_t pack_records(Ctx &c, const sph_state &s, cudaStream_t st);
-cudaError_t scan_exclusive_int(Ctx &c, const int *in, int *out, int n, int *total_dev,
-                               cudaStream_t st);
 // test hook: a sort pass whose look-back predecessor never publishes
 cudaError_t sort_lookback_probe(Ctx &c, int spin_cap, cudaStream_t st);
 // nlist.cu

@@ -724,12 +724,6 @@ static cudaError_t scan_mode(Ctx &c, const int *in, int *out, int n, int mode, i
     return cudaGetLastError();
 }
 
-cudaError_t scan_exclusive_int(Ctx &c, const int *in, int *out, int n, int *total_dev,
-                               cudaStream_t st)
-{
-    return scan_mode(c, in, out, n, 0, total_dev, st);
-}
-
 // -------------------------------------------------------------------- chop
 // Shared leading digits of the keys of slots a and b; -1 when the slots
 // belong to different instances of a batch (inst != nullptr): instances never

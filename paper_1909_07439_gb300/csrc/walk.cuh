@@ -290,35 +290,6 @@ __device__ bool walk_group(const WalkTree &T, int root, float4 glo, float4 ghi, 
     return ok;
 }
 
-// Walk the tree below `root` for the box [glo, ghi] in force mode and store
-// every opened leaf as (node, first particle) in out[0 .. cap).  Returns the
-// number of leaves, or -1 if they did not fit or the stack overflowed.
-__device__ __forceinline__ int walk_leaves(const WalkTree &T, int root, float4 glo, float4 ghi,
-                                           float hgroup, float node_scale, WalkSmem &sm, int2 *out,
-                                           int cap)
-{
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = lane_lt();
-    bool ok = true;
-    int sp = 1, nout = 0;
-    if (lane == 0) sm.stk[0] = make_int2(root, 1);
-    __syncwarp();
-    while (sp > 0) {
-        bool leaf;
-        int2 ref;
-        int node;
-        walk_step(T, glo, ghi, 0.f, true, hgroup, node_scale, sm, sp, ok, leaf, ref, node);
-        const unsigned bleaf = __ballot_sync(0xffffffffu, leaf);
-        if (leaf) {
-            const int p = nout + __popc(bleaf & lt);
-            if (p < cap) out[p] = make_int2(node, ref.x);
-        }
-        nout += __popc(bleaf);
-        __syncwarp();
-    }
-    return ok && nout <= cap ? nout : -1;
-}
-
 // Shared memory of a wide walk: W nodes per lane and step.
 template <int W, int STK>
 struct WalkSmemW {
@@ -326,10 +297,11 @@ struct WalkSmemW {
     int nodes[32 * W];
 };
 
-// walk_leaves with W nodes tested per lane and step (fewer, wider steps: the
-// node loads of a step are independent, so a step costs about one memory
-// latency whatever W is).  Same opening test and result set as walk_leaves;
-// the order of `out` differs.
+// Walk the tree below `root` for the box [glo, ghi] in force mode and store every
+// opened leaf as (node, first particle) in out[0 .. cap), in no particular order.
+// Returns the number of leaves, or -1 if they did not fit or the stack overflowed.
+// W nodes are tested per lane and step: the node loads of a step are independent,
+// so a step costs about one memory latency whatever W is.
 template <int W, int STK, bool PER = true>
 __device__ __forceinline__ int walk_leaves_wide(const WalkTree &T, int root, float4 glo, float4 ghi,
                                                 float hgroup, float node_scale, WalkSmemW<W, STK> &sm,
