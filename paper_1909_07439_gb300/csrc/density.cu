@@ -843,6 +843,8 @@ cudaError_t density_lists(Ctx &c, const sph_state &s, const sph_params &p, cudaS
 cudaError_t density_solve(Ctx &c, const sph_state &s, const sph_params &p, cudaStream_t st,
                           const Batch *batch)
 {
+    if (!c.work_zeroed) return cudaErrorInvalidValue;  // without it every group would be skipped
+    c.work_zeroed = false;
     DensArgs a{};
     a.inst = batch ? c.inst : nullptr;
     a.h_in_scale = 1.f + kPad;
@@ -881,7 +883,6 @@ cudaError_t density_solve(Ctx &c, const sph_state &s, const sph_params &p, cudaS
     a.fixed_iters = p.density_iters;
     a.err = c.d_err;
     a.counters = c.d_counters;
-    // (the list build zeroed the work counters)
     if (p.kernel == 1) return density_solve_k<1>(c, a, p, st);
     if (p.kernel == 2) return density_solve_k<2>(c, a, p, st);
     return density_solve_k<0>(c, a, p, st);

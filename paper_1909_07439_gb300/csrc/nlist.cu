@@ -543,7 +543,9 @@ cudaError_t nlist_pass(Ctx &c, const sph_state &s, const sph_params &p, float pa
     e = clear_words(Clear{{c.tree.rec_ctl, c.tree.rec_bad, c.d_sizes + SZ_NL}, {2, batch ? batch->n_inst : 1, 2}}, st);
     if (e != cudaSuccess) return e;
     const NlistArgs a = nlist_args(c, s, p, pad, batch);
-    return launch_nlist(c, a, blocks, st);
+    e = launch_nlist(c, a, blocks, st);
+    c.work_zeroed = e == cudaSuccess;
+    return e;
 }
 
 cudaError_t check_list_kernel(Ctx &c, const sph_params &p, cudaStream_t st)

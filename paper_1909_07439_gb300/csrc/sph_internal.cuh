@@ -130,6 +130,9 @@ struct Ctx {
     int *nl_len = nullptr;
     int nl_stride = 128;
     int nl_kernel = -1;
+    // the last list build zeroed the work counters of the density kernels, and no
+    // density pass has used them since
+    bool work_zeroed = false;
     // Inside a step the force pass writes drho/dt (its pressure-work sum is
     // the same sum up to a per-particle factor) and the density pass gathers
     // positions only; standalone density passes write drho/dt themselves.
