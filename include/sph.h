@@ -67,7 +67,8 @@ typedef struct {
     int32_t n_group;     /* max particles per walk group (1..32)                        */
     int32_t tile;        /* shared-memory list capacity per target of the walking
                             fallback kernels, 0 = default (density 96 for M4, 192
-                            for M6, 128 for C6; force 96 for M4, else 128)     */
+                            for M6, 128 for C6, up to 384 with hfact; force 96
+                            for M4, else 128)                                  */
     int32_t max_h_iter;  /* Newton iteration cap (>= 1)                                 */
     int32_t density_iters; /* 0: iterate to h_tol; k > 0: exactly k updates (Sect. 3.2.1) */
     /* Launch shape of the neighbour-list density and force kernels (results

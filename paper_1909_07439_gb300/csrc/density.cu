@@ -21,6 +21,8 @@
 // lane = t * L + sub; partial sums are reduced across the L lanes with xor
 // shuffles, so every lane of a target holds the full sums and takes the
 // same Newton step.
+#include <algorithm>
+
 #include "kernels.cuh"
 #include "walk.cuh"
 
@@ -73,6 +75,7 @@ struct DensArgs {
     float h_in_scale; // 1 + pad
     float hfact, tol, gamma;
     int tb;           // targets per batch of the list kernel (4, 8 or 16)
+    int n;            // particles
     int vd;           // 1: drho/dt here (Eq. 3); 0: the force pass of the step writes it
     int max_iter, fixed_iters;
     int *err;
@@ -343,14 +346,14 @@ __global__ void __launch_bounds__(256, 4) density_list_kernel(DensArgs a)
 // it had reached there, whose first updates are the largest, with its bracket and
 // its count of updates (a fixed number of updates starts over from the starting
 // h).  Bound by the latency of its walks: a warp's next candidates are loaded
-// while it tests the ones before, its batches have 4 targets, and lists that
-// overflow are summed while walking in that sweep only.  Density stage, before (from the starting
-// h, whole batches, no prefetch, streaming for good) and now: 8192 particles
-// from a rough h (1248 batches) 262 -> 161 us, the M6 tube (76 batches past the
-// list capacity) 392 -> 323 us.  List pads of 6 and 10 % instead of 3 were no
-// faster (163 and 209 us for the sphere).
-template <int CAP, int K>
-__global__ void __launch_bounds__(kDensWarps * 32, 4) density_walk_kernel(DensArgs a)
+// while it tests the ones before, its batches have 4 targets, lists that overflow
+// are summed while walking in that sweep only, and lists that would overflow again
+// are built without the pad.  The density stage of a sphere from 0.9 times its h
+// (8192 particles) or 0.7 times (30 k, 500 k), before (from the starting h, batches of
+// 8, no prefetch, streaming for good) and now: 200 -> 116 us, 494 -> 374 us, 4.44 ->
+// 4.13 ms.  List pads of 6 and 10 % instead of 3 were no faster.
+template <int CAP, int K, int BLOCKS>
+__global__ void __launch_bounds__(kDensWarps * 32, BLOCKS) density_walk_kernel(DensArgs a)
 {
     pdl_sync();
     extern __shared__ __align__(16) unsigned char dsm_raw[];
@@ -397,6 +400,7 @@ __global__ void __launch_bounds__(kDensWarps * 32, 4) density_walk_kernel(DensAr
             float hw = h * (1.f + kPad);  // list radius is R hw
             bool valid = false;               // lists cover the current h
             bool streamed = false;            // batch overflowed the tile
+            bool exact = false;               // lists without the pad
             bool conv = !on;
             int it = __float_as_int(from.w);  // the same for the targets of a batch
             bool final_pass = !fixed && it >= limit;  // the last update left the pad
@@ -423,7 +427,7 @@ __global__ void __launch_bounds__(kDensWarps * 32, 4) density_walk_kernel(DensAr
                 };
                 if (!valid) {
                     // (re)build the candidate lists with a walk
-                    hw = h * (1.f + kPad);
+                    hw = exact ? h : h * (1.f + kPad);
                     const float myr = SphKernel<K>::R * hw;
                     if (act && sub == 0) sm.tr2[t] = myr * myr;
                     if (lane < kTB) sm.tlen[lane] = 0;
@@ -518,10 +522,14 @@ __global__ void __launch_bounds__(kDensWarps * 32, 4) density_walk_kernel(DensAr
                     ++n_newton;
                 }
                 if (final_pass) break;
+                const float h_was = h;
                 if (on && !conv) {
                     newton_update(h, hlo, hhi, conv, s0, s1, M, fixed, a.tol, SphKernel<K>::C);
                     if (h > hw) valid = false;  // outgrew the padded list
                 }
+                // lists that would not hold the pad at the new h either
+                const float grown = (1.f + kPad) * (h / h_was);
+                exact = __any_sync(0xffffffffu, act && !valid && cf * (grown * grown * grown) > CAP);
                 ++it;
                 if (__any_sync(0xffffffffu, !valid)) valid = false;
                 if (fixed) {
@@ -701,7 +709,7 @@ __global__ void list_set_kernel(const float4 *__restrict__ pos, const float *__r
 
 // ------------------------------------------------------------------ host side
 // one-time kernel attributes and occupancy (also called before graph capture)
-template <int CAP, int K>
+template <int CAP, int K, int BLOCKS = 4>
 static cudaError_t configure_density(int &blocks)
 {
     static std::mutex mu;  // first calls may come from several host threads
@@ -710,11 +718,11 @@ static cudaError_t configure_density(int &blocks)
     static int nb_cached = 1;
     if (!configured) {
         size_t smem = sizeof(DensSmem<CAP>) * kDensWarps;
-        cudaError_t e = cudaFuncSetAttribute(density_walk_kernel<CAP, K>,
+        cudaError_t e = cudaFuncSetAttribute(density_walk_kernel<CAP, K, BLOCKS>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         int nb = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, density_walk_kernel<CAP, K>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, density_walk_kernel<CAP, K, BLOCKS>,
                                                           kDensWarps * 32, smem);
         if (e != cudaSuccess) return e;
         nb_cached = nb > 0 ? nb : 1;
@@ -758,14 +766,15 @@ static cudaError_t configure_density_list(int blocks[4])
     return cudaSuccess;
 }
 
-template <int CAP, int K>
+template <int CAP, int K, int BLOCKS = 4>
 static cudaError_t launch_density_walk(Ctx &c, const DensArgs &a, cudaStream_t st)
 {
     int blocks = 1;
-    cudaError_t e = configure_density<CAP, K>(blocks);
+    cudaError_t e = configure_density<CAP, K, BLOCKS>(blocks);
     if (e != cudaSuccess) return e;
     size_t smem = sizeof(DensSmem<CAP>) * kDensWarps;
-    launch(density_walk_kernel<CAP, K>, c.num_sms * blocks, kDensWarps * 32, smem, st, a);
+    const int grid = std::min(c.num_sms * blocks, div_up(a.n, kDensWarps));  // a warp per item, n items at most
+    launch(density_walk_kernel<CAP, K, BLOCKS>, grid, kDensWarps * 32, smem, st, a);
     return cudaGetLastError();
 }
 
@@ -775,10 +784,17 @@ static cudaError_t configure_density_k()
     int b, bl[4];
     cudaError_t e = configure_density_list<K>(bl);
     if (e == cudaSuccess) e = configure_density<64, K>(b);
+    if (e == cudaSuccess) e = configure_density<64, K, 5>(b);
     if (e == cudaSuccess) e = configure_density<80, K>(b);
+    if (e == cudaSuccess) e = configure_density<80, K, 5>(b);
     if (e == cudaSuccess) e = configure_density<96, K>(b);
+    if (e == cudaSuccess) e = configure_density<96, K, 5>(b);
     if (e == cudaSuccess) e = configure_density<128, K>(b);
+    if (e == cudaSuccess) e = configure_density<128, K, 5>(b);
     if (e == cudaSuccess) e = configure_density<192, K>(b);
+    if (e == cudaSuccess) e = configure_density<192, K, 5>(b);
+    if (e == cudaSuccess) e = configure_density<256, K>(b);
+    if (e == cudaSuccess) e = configure_density<384, K>(b);
     return e;
 }
 
@@ -817,15 +833,27 @@ static cudaError_t density_solve_k(Ctx &c, DensArgs &a, const sph_params &p, cud
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // default tile: the mean density set (about 58 for M4 at hfact 1.2, 82 and
-    // 113 for M6 at 0.9 and 1.0, 74 for Wendland C6 at 1.3) within the pad, with
-    // room to spare: an overflow costs a walk in every sweep
+    // Default tile: the lists of a uniform cloud (58 entries for M4 at hfact 1.2, 82
+    // and 113 for M6 at 0.9 and 1.0, 74 for Wendland C6 at 1.3) within the pad, with a
+    // quarter to spare, since an overflow costs a walk in every sweep: at hfact 1.5
+    // and 1.8, 500 k particles all walked, the M4 density stage takes 2.9 and 8.6 ms,
+    // with tiles of 96 6.8 and 12.2 ms.  Beyond 384 entries lists that large leave
+    // too few warps (hfact 2.5: 38 ms against 19 ms streamed through a tile of 96).
+    // Where the lists do not fit, five blocks per SM (95 registers) hide more of the
+    // walks: hfact 2.5 21.0 -> 18.6 ms; where they fit, four (109 registers), since a
+    // few batches wait for one chain: 8192 particles 116 us against 118.
+    const float rl = SphKernel<K>::R * p.hfact * (1.f + kPad);
+    const float mean = 4.18879f * rl * rl * rl;
     int cap = p.tile > 0 ? p.tile : K == 0 ? 96 : K == 1 ? 192 : 128;
-    if (cap <= 64) return launch_density_walk<64, K>(c, a, st);
-    if (cap <= 80) return launch_density_walk<80, K>(c, a, st);
-    if (cap <= 96) return launch_density_walk<96, K>(c, a, st);
-    if (cap <= 128) return launch_density_walk<128, K>(c, a, st);
-    return launch_density_walk<192, K>(c, a, st);
+    if (p.tile == 0 && 1.25f * mean <= 384.f) cap = std::max(cap, (int)(1.25f * mean));
+    const bool many = mean > (float)cap;
+    if (cap <= 64) return many ? launch_density_walk<64, K, 5>(c, a, st) : launch_density_walk<64, K>(c, a, st);
+    if (cap <= 80) return many ? launch_density_walk<80, K, 5>(c, a, st) : launch_density_walk<80, K>(c, a, st);
+    if (cap <= 96) return many ? launch_density_walk<96, K, 5>(c, a, st) : launch_density_walk<96, K>(c, a, st);
+    if (cap <= 128) return many ? launch_density_walk<128, K, 5>(c, a, st) : launch_density_walk<128, K>(c, a, st);
+    if (cap <= 192) return many ? launch_density_walk<192, K, 5>(c, a, st) : launch_density_walk<192, K>(c, a, st);
+    if (cap <= 256) return launch_density_walk<256, K>(c, a, st);
+    return launch_density_walk<384, K>(c, a, st);
 }
 
 cudaError_t density_lists(Ctx &c, const sph_state &s, const sph_params &p, cudaStream_t st,
@@ -860,6 +888,7 @@ cudaError_t density_solve(Ctx &c, const sph_state &s, const sph_params &p, cudaS
     a.vel = (const float4 *)s.vel;
     a.rec = c.rec;
     a.vd = c.drhodt_in_force ? 0 : 1;
+    a.n = (int)s.n;
     a.h = s.h;
     a.reached = c.tmp4[3];  // free between the tree build and the adjoint
     a.rho = s.rho;
