@@ -3,6 +3,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "sph_internal.cuh"
@@ -10,6 +11,15 @@
 using namespace sph;
 
 namespace {
+
+// Held while a step's graph is recorded and by the calls that wait for the whole
+// device (a context's creation and destruction, the tree's and the counters'
+// export): such a wait in another thread would invalidate the recording, and fail.
+std::recursive_mutex &device_wide()
+{
+    static std::recursive_mutex m;
+    return m;
+}
 
 const char *status_text(sph_status s)
 {
@@ -291,6 +301,7 @@ sph_status record_step_graph(Ctx &c, Ctx::StepGraph &g, const sph_state &s, cons
     cudaStream_t cs = c.capture_stream;
     c.capture_ev.clear();
     for (auto &x : c.capture_launches) x = 0;
+    std::lock_guard<std::recursive_mutex> lock(device_wide());
     CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal), "begin capture");
     c.capturing = true;
     const sph_status r = enqueue_step(c, s, p, d_dt, d_time, cs, out);
@@ -370,6 +381,7 @@ sph_status sph_create(sph_ctx **out, int64_t max_n, int device)
     if (!out) return SPH_ERR_INVALID_ARG;
     *out = nullptr;
     if (max_n < 1 || max_n >= (int64_t)1 << 31) return SPH_ERR_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> lock(device_wide());
     sph_ctx *h = new (std::nothrow) sph_ctx();
     if (!h) return SPH_ERR_NOMEM;
     Ctx &c = h->impl;
@@ -463,6 +475,7 @@ sph_status sph_create(sph_ctx **out, int64_t max_n, int device)
 void sph_destroy(sph_ctx *h)
 {
     if (!h) return;
+    std::lock_guard<std::recursive_mutex> lock(device_wide());
     Ctx &c = h->impl;
     cudaSetDevice(c.device);
     cudaDeviceSynchronize();
@@ -861,6 +874,7 @@ sph_status sph_batch_step(sph_ctx *h, sph_state *s, const int64_t *d_offsets, in
         if (!c.capture_stream)
             CK(cudaStreamCreateWithFlags(&c.capture_stream, cudaStreamNonBlocking), "capture stream");
         cudaStream_t cs = c.capture_stream;
+        std::lock_guard<std::recursive_mutex> lock(device_wide());
         CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal), "begin capture");
         cudaError_t e = enqueue_batch_step(c, *s, *p, b, d_dt, d_time, cs);
         cudaGraph_t g = nullptr;
@@ -942,6 +956,7 @@ sph_status sph_get_tree(sph_ctx *h, int32_t *h_level, int32_t *h_first, int32_t 
     if (!h || !n_nodes || !n_groups) return SPH_ERR_INVALID_ARG;
     Ctx &c = h->impl;
     int sz[SZ_N];
+    std::lock_guard<std::recursive_mutex> lock(device_wide());
     CK(cudaDeviceSynchronize(), "tree sync");
     CK(cudaMemcpy(sz, c.d_sizes, sizeof(sz), cudaMemcpyDeviceToHost), "sizes copy");
     *n_nodes = sz[SZ_NODES];
@@ -981,6 +996,7 @@ sph_status sph_get_stats(sph_ctx *h, sph_stats *out)
     Ctx &c = h->impl;
     unsigned long long v[C_N];
     int sz[SZ_N];
+    std::lock_guard<std::recursive_mutex> lock(device_wide());
     CK(cudaDeviceSynchronize(), "stats sync");
     CK(cudaMemcpy(v, c.d_counters, sizeof(v), cudaMemcpyDeviceToHost), "stats copy");
     CK(cudaMemcpy(sz, c.d_sizes, sizeof(sz), cudaMemcpyDeviceToHost), "sizes copy");
