@@ -70,6 +70,9 @@ class _Evaluate(torch.autograd.Function):
     @staticmethod
     def backward(fctx, gh, grho, gom, gacc):
         pos, velu, h0, alpha, perm, h, rho, omega = fctx.saved_tensors
+        # the library takes raw pointers; a saved-tensor hook may return anything
+        if not all(t.is_cuda for t in (pos, velu, perm, h, rho, omega)):
+            raise TypeError("evaluate's saved tensors must be on the GPU")
         handle, p = fctx.handle, fctx.p
         n, dev = pos.shape[0], pos.device
         perm = perm.long()
@@ -80,13 +83,13 @@ class _Evaluate(torch.autograd.Function):
         # forward's rho and Omega in place of that sweep's.  The adjoint passes
         # read nothing of a force pass.
         s = DeviceState(n, device=dev, zero=False)
-        s.pos, s.vel = pos.detach().index_select(0, perm), velu.detach().index_select(0, perm)
+        s.pos, s.vel = (t.detach().to(torch.float32).index_select(0, perm) for t in (pos, velu))
         s.h.copy_(h)
         q = _params(p, p.alpha_av)
         q.density_iters, q.h_tol = 0, 4.0
         native.sph_build_tree(handle, s.c, p)
         native.sph_density(handle, s.c, q)
-        s.rho, s.omega = rho, omega
+        s.rho, s.omega = (t.to(torch.float32).contiguous() for t in (rho, omega))
 
         def to_curve(g, shape):
             return (torch.zeros(shape, dtype=torch.float32, device=dev) if g is None

@@ -110,3 +110,31 @@ def test_gradients_match_fp64_autograd(lib, n, kernel, iters):
     off = abs(float(al.grad) - float(t.sum())) / float(t.norm())
     print(f"n {n} kernel {kernel} iters {iters}: dL/dalpha off by {off:.1e} of the terms' norm")
     assert off < 7e-6
+
+
+def test_backward_again_and_through_saved_tensor_hooks(lib):
+    native, ctx = lib
+    w, g = _cloud(1200, 8, R.M4)
+    p = native.sph_params_default()
+    cot = torch.tensor(g, device="cuda")
+
+    def grads(hooks, times):
+        with hooks:
+            pos, vel, al, out = _evaluate(ctx, w, p)
+        out[0].mul_(2.0)    # the outputs are the caller's
+        for k in range(times):
+            for t in (pos, vel, al):
+                t.grad = None
+            torch.autograd.backward(out[3], cot, retain_graph=k + 1 < times)
+        return pos.grad, vel.grad, al.grad
+
+    plain = lambda t: t  # noqa: E731
+    want = grads(torch.autograd.graph.saved_tensors_hooks(plain, plain), 1)
+    for hooks, times in ((torch.autograd.graph.saved_tensors_hooks(plain, plain), 2),
+                         (torch.autograd.graph.save_on_cpu(pin_memory=True), 1),
+                         (torch.autograd.graph.saved_tensors_hooks(lambda t: t.double(), plain), 1)):
+        got = grads(hooks, times)
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+        assert abs(float(got[2]) / float(want[2]) - 1) < 1e-12     # FP64 sum in any order
+    with pytest.raises(TypeError):
+        grads(torch.autograd.graph.saved_tensors_hooks(lambda t: t.cpu(), plain), 1)
