@@ -62,13 +62,13 @@ FLOP_PAIR = {0: (FLOP_FORCE_PAIR, FLOP_DENSITY_PAIR), 1: (106, 75), 2: (104, 66)
 EXEC_FLOP_FORCE_PAIR = 85.4
 # DRAM bytes (read + write) per launch of the pair kernels from one ncu capture
 # of the 128^3 step; None where the kernel changed after the capture.
-NCU_TRAFFIC = {"nlist_kernel": 136.681472e6 + 586.587904e6,
-               "density_list_kernel": 928.414208e6 + 117.061888e6,
-               "force_list_kernel": 966.498304e6 + 34.54592e6}
+NCU_TRAFFIC = {"nlist_kernel": 137.022464e6 + 586.684672e6,
+               "density_list_kernel": 928.51328e6 + 117.110272e6,
+               "force_list_kernel": 965.879296e6 + 34.175232e6}
 # Issue slots busy (smsp__issue_active, fraction of the active cycles) in the
 # same ncu captures: the list build is bound by instruction issue, which its
 # FP32 fraction (8 FLOP per candidate test) does not show.
-NCU_ISSUE_ACTIVE = {"nlist_kernel": 0.758, "density_list_kernel": 0.659, "force_list_kernel": 0.641}
+NCU_ISSUE_ACTIVE = {"nlist_kernel": 0.756, "density_list_kernel": 0.655, "force_list_kernel": 0.638}
 # Self-gravity FP32 operations per interaction (softened pair: separation 3,
 # r^2 + eps^2 6, the inverse powers 3, m/r and m/r^3 2, acceleration 6,
 # potential 1 = 21; quadrupole cell: the same 20 plus Q d 15, d.Q.d 5, the
